@@ -8,10 +8,12 @@
 //                        nodes[2i] (lo) and nodes[2i+1] (hi), so the two children of
 //                        node i sit in one aligned 64-byte line nodes[4i .. 4i+3].
 //                        Leaf l is node L + l; empty buckets have an inverted box.
-//   obb   float4[4L]     oriented box of every bucket (same allocation, after the
-//                        nodes): centre c and half-extents h along three orthonormal
+//   obb   float4[4W]     oriented box of every bucket and of every third level above
+//                        the buckets (W = wide_leaf(L) + L rounded up to eights, same
+//                        allocation, after the nodes): centre c and half-extents h along three orthonormal
 //                        axes a_k fitted to the bucket's points, as
-//                        (c, h0) (a0, h1) (a1, h2) (a2, r), r the bucket's radius
+//                        (c, h0) (a0, h1) (a1, h2) (a2, r), r the bucket's radius;
+//                        eight boxes together, one float4 of each at a time (obb_at)
 //   src   float4[M]      source points in Morton order, .w = original index bits
 //   PairState            one registration's solver state (FP64), ~2 KB
 //   partial double[T][K] per-tile reduction records (T = ceil(M / kBlock) tiles)
@@ -72,7 +74,9 @@ struct Index {
     const ushort4 *pts16;   // FP16 storage (x, y, z as half offsets in the bucket box), or null
     int n;
     int L;
-    const float4 *obb;      // oriented bucket boxes (4 float4 per bucket), or null: axis-aligned boxes only
+    const float4 *obb;      // oriented boxes of the buckets and of every third level above them
+    int first;              // wide_first(L)
+    int leaf0;              // wide_leaf(L)
 };
 
 enum Phase : int {
@@ -254,8 +258,16 @@ __device__ __forceinline__ float box_d2(float4 lo, float4 hi, const float xh[3],
 // window.
 constexpr float kObbShrink = 1.0f - 2e-5f;
 
+// Oriented box w of the array: its four float4 are 8 apart (eight boxes are
+// stored together, first all their centres, then each axis: eight lanes testing
+// a node's eight children then read whole 128-byte lines).
+template <class T>
+__device__ __forceinline__ T *obb_at(T *obb, int w) {
+    return obb + ((size_t)(w >> 3) * 32 + (w & 7));
+}
+
 __device__ __forceinline__ float obb_d2(const float4 *o, const float xh[3], const float xl[3]) {
-    return obb_eval(__ldg(o), __ldg(o + 1), __ldg(o + 2), __ldg(o + 3), xh, xl);
+    return obb_eval(__ldg(o), __ldg(o + 8), __ldg(o + 16), __ldg(o + 24), xh, xl);
 }
 
 // Box test of a search lane: xdn <= x <= xup on every axis, so lo - xup and
@@ -372,8 +384,8 @@ __device__ __forceinline__ bool nn_offer(NNLane &q, float4 p, int j) {
 // storage decodes points inside the axis-aligned box only, so it skips this test.
 template <int PREC = PREC_FP64>
 __device__ __forceinline__ bool obb_meets(const Index &ix, const NNLane &q, int leaf) {
-    if (PREC == PREC_FP16 || ix.obb == nullptr) return true;
-    return obb_d2(ix.obb + 4 * (leaf - ix.L), q.xh, q.xl) * kObbShrink <= q.bestf;
+    if (PREC == PREC_FP16) return true;
+    return obb_d2(obb_at(ix.obb, leaf - ix.L + ix.leaf0), q.xh, q.xl) * kObbShrink <= q.bestf;
 }
 
 // Depth-first search from the root with the lane's current bound (q.bestf).
@@ -735,6 +747,225 @@ __device__ __forceinline__ bool halfwarp_nn(const Index &ix, NNLane &q, int *stk
 }
 
 // ---------------------------------------------------------------------------
+// Group search: kGroup lanes per query, 32 / kGroup queries per warp. The binary
+// box tree is walked three levels at a time: the eight descendants of a node
+// three levels down are nodes 8 i .. 8 i + 7, and each lane of the group tests
+// kGroupC of their boxes. A tree whose depth is not a multiple of three starts
+// with the remainder (2 or 4 nodes).
+//   - inner nodes: the nearest child within the bound is entered at once, the
+//     others are pushed with their distance on the group's stack;
+//   - buckets are scanned nearest first, the lanes sharing the points, and the
+//     group's bound (and with it the buckets still waiting) is refreshed after
+//     each;
+//   - a pop looks at the top kGroup entries together and drops those the bound
+//     has overtaken.
+// The set of points offered is every point that can beat the bound, so the
+// result is the exact argmin of the serial search, ties included. All 32 lanes
+// run every warp-wide primitive; a group without a query (`live` false) only
+// takes part in them. A path holds at most kGroupDepth inner levels, each
+// leaving at most seven entries, so the stack cannot overflow.
+//
+// The boxes tested are the oriented ones, at every level (wide_box): on a
+// surface an axis-aligned box of a tilted patch is as thick as the patch is
+// wide, and a query a little off the surface is inside the boxes of all the
+// patches around it. FP16 storage decodes points inside the axis-aligned boxes
+// only, so it tests those.
+//
+// What bounds it: issue slots (63% busy) and the L1 latency of each round's
+// loads; about 95 instructions a round and 60 a bucket, 16 rounds and 8 buckets
+// for four warm-started queries that stay together. Measured (ellipsoids,
+// N = 500,000, M = 200,000, FP64, mean over a registration's passes): two
+// queries per warp over the axis-aligned boxes 357 us, this 196 us; with four
+// lanes per query (two children each) 206 us, with two 364 us before the boxes
+// were stored in eights (the L1 then serves whole lines: 377 -> 335 us); the
+// oriented boxes above the buckets take the rounds per query from 20.5 to 14.8.
+// ---------------------------------------------------------------------------
+constexpr int kGroup = 8;                         // lanes per query
+constexpr int kGroupQ = 32 / kGroup;              // queries per warp
+constexpr int kGroupC = 8 / kGroup;               // children per lane
+constexpr int kGroupDepth = 9;                    // inner levels of a tree over 2^30 points: ceil(26 / 3)
+constexpr int kGroupStack = 7 * kGroupDepth + 1;  // stack entries per group
+constexpr unsigned kGroupMask = (1u << kGroup) - 1u;
+
+// Order of the oriented boxes: level by level from the top, each a multiple of
+// three above the buckets; the first level has wide_first(L) nodes, at positions
+// 8 - wide_first(L) .. 7 (empty boxes before them), and the children of the node
+// at position p are at wide_child(first, p) .. + 7. Buckets start at wide_leaf(L).
+FRICP_HD inline int wide_first(int L) {
+    int depth = 0;
+    while ((1 << depth) < L) ++depth;
+    return 1 << (depth == 0 ? 0 : (depth - 1) % 3 + 1);
+}
+FRICP_HD inline int wide_pos(int first, int level_size) { return (level_size - first) / 7 + 8 - first; }
+FRICP_HD inline int wide_leaf(int L) { return wide_pos(wide_first(L), L); }
+FRICP_HD inline int wide_child(int first, int p) { return 8 * p + 8 * first - 56; }
+
+// Walk the tree for the point x = xh + xl of this group, offering every point of
+// every bucket within `bound` to `offer(j, p)`, which returns the smallest float
+// distance this lane was offered so far.
+template <int PREC, class Offer>
+__device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], const float xl[3], float &bound,
+                                           float2 *stk, bool live, Offer offer) {
+    constexpr bool AABB = PREC == PREC_FP16;
+    const unsigned FULL = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000), OUT = __int_as_float(0x7fc00000);   // OUT: not within any bound
+    const int lane = threadIdx.x & 31;
+    const int gl = lane & (kGroup - 1);
+    const int gs = lane & ~(kGroup - 1);
+    const unsigned below = (1u << gl) - 1u;
+    const int leaf0 = AABB ? ix.L : ix.leaf0;     // first bucket: as a node of the binary tree, or a position
+    int base = AABB ? ix.first : 0;               // first of the eight boxes this round tests
+    int cnt = live ? (AABB ? ix.first : 8) : 0;   // how many of them (eight after the first round)
+    int sp = 0;
+    while (__any_sync(FULL, cnt != 0)) {
+        const bool leaf = AABB ? base >= leaf0 : base + 7 >= leaf0;
+        float key[kGroupC];
+        unsigned near = 0xffffffffu;
+#pragma unroll
+        for (int c = 0; c < kGroupC; ++c) {
+            const int g = gl + c * kGroup;
+            key[c] = OUT;
+            if (AABB ? g < cnt : cnt != 0) {
+                if (AABB)
+                    key[c] = box_d2(__ldg(ix.nodes + 2 * (base + g)), __ldg(ix.nodes + 2 * (base + g) + 1), xh, xl) *
+                             kShrink;
+                else
+                    key[c] = obb_d2(ix.obb + ((size_t)(base >> 3) * 32 + g), xh, xl) * kObbShrink;
+                if (key[c] <= bound) near = min(near, (__float_as_uint(key[c]) & ~7u) | g);
+                else key[c] = OUT;
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < kGroup; o <<= 1) near = min(near, __shfl_xor_sync(FULL, near, o));
+        const bool any = near != 0xffffffffu;
+        int w = near & 7;
+        int node = -1;
+        if (any && !leaf) node = base + w;   // enter the nearest, push the others
+#pragma unroll
+        for (int c = 0; c < kGroupC; ++c) {
+            const int g = gl + c * kGroup;
+            const bool push = any && !leaf && key[c] <= bound && g != w;
+            const unsigned m = (__ballot_sync(FULL, push) >> gs) & kGroupMask;
+            if (push) stk[sp + __popc(m & below)] = make_float2(key[c], __int_as_float(base + g));
+            sp += __popc(m);
+        }
+        bool scan = any && leaf;
+        while (__any_sync(FULL, scan)) {   // the nearest bucket, then the others that stay within the bound
+            float d = INF;
+            if (scan) {
+                const int j0 = (base + w - leaf0) * kLeaf + gl;
+#pragma unroll
+                for (int t = 0; t < kLeaf / kGroup; ++t) {
+                    const int j = j0 + t * kGroup;
+                    if ((unsigned)j < (unsigned)ix.n) d = offer(j, target_point<PREC>(ix, j));
+                }
+            }
+            bound = fminf(bound, d);
+#pragma unroll
+            for (int o = 1; o < kGroup; o <<= 1) bound = fminf(bound, __shfl_xor_sync(FULL, bound, o));
+            unsigned m = 0;
+#pragma unroll
+            for (int c = 0; c < kGroupC; ++c) {
+                if (gl + c * kGroup == w) key[c] = OUT;
+                m |= ((__ballot_sync(FULL, scan && key[c] <= bound) >> gs) & kGroupMask) << (c * kGroup);
+            }
+            scan = m != 0u;
+            w = __ffs(m) - 1;
+        }
+        __syncwarp();
+        while (__any_sync(FULL, node < 0 && sp > 0)) {   // pop
+            const int k = min(kGroup, sp);
+            const float2 e = gl < k ? stk[sp - 1 - gl] : make_float2(OUT, 0.0f);
+            const unsigned ok = (__ballot_sync(FULL, e.x <= bound) >> gs) & kGroupMask;
+            const int f = __ffs(ok) - 1;
+            const int top = __shfl_sync(FULL, __float_as_int(e.y), gs + max(f, 0));
+            if (node < 0) {
+                sp -= ok ? f + 1 : k;
+                if (ok) node = top;
+            }
+        }
+        __syncwarp();
+        cnt = node < 0 ? 0 : 8;
+        base = AABB ? 8 * node : 8 * node + 8 * ix.first - 56;
+    }
+}
+
+__device__ __forceinline__ float point_d2f(const float xh[3], const float xl[3], float4 p) {
+    const float dx = (xh[0] - p.x) + xl[0];
+    const float dy = (xh[1] - p.y) + xl[1];
+    const float dz = (xh[2] - p.z) + xl[2];
+    return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+}
+
+// Closest point of a group's query: its bucket-order index, or -1 if no target
+// point lies within `bound` (a squared float distance; the distance to a known
+// target point for a warm start).
+//
+// The walk ranks by float distance only: each lane keeps its nearest point and
+// the distance of its second nearest. Unless another point lies within the tie
+// window of the smallest float distance, the nearest is the winner; ties inside
+// the window are ranked as the serial search ranks them, by double-float distance
+// and original index, over the lanes' nearest points, or, when a lane has seen
+// two such points, by a second walk within the window.
+template <int PREC>
+__device__ __forceinline__ int group_nn(const Index &ix, const float xh[3], const float xl[3], float bound,
+                                        float2 *stk, bool live) {
+    const unsigned FULL = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31;
+    const int gs = lane & ~(kGroup - 1);
+    const float limit = PREC == PREC_FP64 ? bound * kTieWindow : bound;
+    float d1 = INF, d2 = INF;
+    int j1 = -1;
+    group_walk<PREC>(ix, xh, xl, bound, stk, live, [&](int j, float4 p) {
+        const float d = point_d2f(xh, xl, p);
+        d2 = fminf(d2, fmaxf(d1, d));
+        if (d < d1) j1 = j;
+        d1 = fminf(d1, d);
+        return d1;
+    });
+    float best = d1;
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) best = fminf(best, __shfl_xor_sync(FULL, best, o));
+    const float win = PREC == PREC_FP64 ? best * kTieWindow : best;
+    const bool found = live && best <= limit && best < INF;
+    const unsigned m1 = (__ballot_sync(FULL, found && d1 <= win) >> gs) & kGroupMask;
+    const unsigned m2 = (__ballot_sync(FULL, found && d2 <= win) >> gs) & kGroupMask;
+    int j = __shfl_sync(FULL, j1, gs + (m1 ? __ffs(m1) - 1 : 0));
+    if (!found) j = -1;
+    const bool tie = m2 != 0u || __popc(m1) > 1;
+    if (__any_sync(FULL, tie)) {   // rare
+        NNLane q;
+        nn_init(q, xh, xl);
+        const bool again = m2 != 0u;
+        if (tie && !again && d1 <= win) nn_seed<PREC>(q, target_point<PREC>(ix, j1), j1);
+        if (__any_sync(FULL, again)) {
+            float bd = win;
+            if (again) q.bestf = best;
+            group_walk<PREC>(ix, xh, xl, bd, stk, again, [&](int jj, float4 p) {
+                nn_offer<PREC>(q, p, jj);
+                return win;
+            });
+        }
+#pragma unroll
+        for (int o = 1; o < kGroup; o <<= 1) {
+            const float oh = __shfl_xor_sync(FULL, q.best_hi, o);
+            const float ol = __shfl_xor_sync(FULL, q.best_lo, o);
+            const int oo = __shfl_xor_sync(FULL, q.best_orig, o);
+            const int oj = __shfl_xor_sync(FULL, q.best_j, o);
+            if (lex_less(oh, ol, oo, q.best_hi, q.best_lo, q.best_orig)) {
+                q.best_hi = oh;
+                q.best_lo = ol;
+                q.best_orig = oo;
+                q.best_j = oj;
+            }
+        }
+        if (tie) j = q.best_j;
+    }
+    return j;
+}
+
+// ---------------------------------------------------------------------------
 // Query tile: a warp holds kTileQ = 8 Morton-adjacent queries, each on a
 // group of four lanes (lane = 4 g + u: query g, sub-lane u; the four lanes of
 // a group carry the same query and the same warm start: the bound is the
@@ -989,7 +1220,7 @@ struct TargetDev {
     int has_normals;
     float4 *pts;
     float4 *nrm;
-    float4 *nodes;    // 4L float4 of boxes, then 4L float4 of oriented bucket boxes (one allocation)
+    float4 *nodes;    // 4L float4 of boxes, then the oriented boxes (one allocation)
     float4 *obb;      // = nodes + 4L
     ushort4 *pts16;   // FP16 storage, built on first use (build_fp16_storage)
     double centroid[3];
@@ -999,7 +1230,9 @@ struct TargetDev {
     double E_Q, H_Q;
 };
 
-inline Index make_index(const TargetDev &t) { return Index{t.pts, t.nrm, t.nodes, t.pts16, (int)t.n, t.L, t.obb}; }
+inline Index make_index(const TargetDev &t) {
+    return Index{t.pts, t.nrm, t.nodes, t.pts16, (int)t.n, t.L, t.obb, wide_first(t.L), wide_leaf(t.L)};
+}
 
 // Per-thread accounting behind fricp_counters (defined in api.cu).
 struct Counters {

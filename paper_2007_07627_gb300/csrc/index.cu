@@ -175,22 +175,160 @@ __global__ void k_leaf_boxes(const float4 *__restrict__ pts, int64_t n, int L, f
     nodes[2 * node + 1] = hi;
 }
 
+// Box of no points: farther than any finite bound.
+__device__ __forceinline__ void empty_obb(float4 *o) {
+    o[0] = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    o[8] = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+    o[16] = make_float4(0.0f, 1.0f, 0.0f, 0.0f);
+    o[24] = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
+}
+
 // Oriented box of every bucket (obb_fit in obb.cuh), the bound obb_d2 tests.
-// Empty buckets get a zero box: their axis-aligned box (inverted) already fails
-// every test.
 __global__ void k_leaf_obb(const float4 *__restrict__ pts, int64_t n, int L, float4 *__restrict__ obb) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= L) return;
-    float4 *o = obb + 4 * (int64_t)l;
+    float4 *o = obb_at(obb, wide_leaf(L) + l);
     const int64_t beg = (int64_t)l * kLeaf;
     const int64_t end = beg + kLeaf < n ? beg + kLeaf : n;
     if (beg >= end) {
-        for (int k = 0; k < 4; ++k) o[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        empty_obb(o);
         return;
     }
     float4 box[4];
     obb_fit(pts + beg, (int)(end - beg), box);
-    for (int k = 0; k < 4; ++k) o[k] = box[k];
+    for (int k = 0; k < 4; ++k) o[8 * k] = box[k];
+}
+
+// Oriented boxes of the patches three, six and nine levels above the buckets (128,
+// 1,024 and 8,192 points), one per NT threads: axes of the points' scatter about the
+// axis-aligned box's middle, extents in float about a float centre. The float
+// rounding of the extents (5.2e-7 of the radius, as in obb_eval) is inside the
+// widening, twice obb_fit's. `shift` = 3, 6 or 9.
+template <int NT>
+__global__ void __launch_bounds__(256) k_patch_obb(const float4 *__restrict__ pts, int64_t n, int L, int shift,
+                                                   const float4 *__restrict__ nodes, float4 *__restrict__ obb) {
+    __shared__ float s_red[8][10];
+    const int tid = threadIdx.x % NT, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int size = L >> shift;
+    const int l = blockIdx.x * (blockDim.x / NT) + threadIdx.x / NT;
+    const bool in = l < size;
+    const int64_t beg = ((int64_t)l * kLeaf) << shift;
+    const int64_t end = beg + (kLeaf << shift) < n ? beg + (kLeaf << shift) : n;
+    const int cnt = in && end > beg ? (int)(end - beg) : 0;
+    const int node = size + l;
+    float4 *o = obb_at(obb, wide_pos(wide_first(L), size) + l);
+    // sum or max over the NT threads of a patch, the same in all of them
+    auto fold = [&](float *v, int k, bool mx) {
+        for (int a = 0; a < k; ++a)
+            for (int off = 16; off > 0; off >>= 1) {
+                const float x = __shfl_xor_sync(0xffffffffu, v[a], off);
+                v[a] = mx ? fmaxf(v[a], x) : v[a] + x;
+            }
+        if (NT > 32) {
+            __syncthreads();
+            if (lane == 0)
+                for (int a = 0; a < k; ++a) s_red[w][a] = v[a];
+            __syncthreads();
+            for (int a = 0; a < k; ++a) {
+                float x = s_red[0][a];
+                for (int ww = 1; ww < 8; ++ww) x = mx ? fmaxf(x, s_red[ww][a]) : x + s_red[ww][a];
+                v[a] = x;
+            }
+        }
+    };
+    float c[3] = {0.0f, 0.0f, 0.0f};
+    if (cnt > 0) {
+        const float4 lo = nodes[2 * node], hi = nodes[2 * node + 1];
+        c[0] = 0.5f * lo.x + 0.5f * hi.x;
+        c[1] = 0.5f * lo.y + 0.5f * hi.y;
+        c[2] = 0.5f * lo.z + 0.5f * hi.z;
+    }
+    float v[9] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    for (int k = tid; k < cnt; k += NT) {
+        const float4 p = pts[beg + k];
+        const float d[3] = {p.x - c[0], p.y - c[1], p.z - c[2]};
+        v[0] += d[0];
+        v[1] += d[1];
+        v[2] += d[2];
+        v[3] = fmaf(d[0], d[0], v[3]);
+        v[4] = fmaf(d[0], d[1], v[4]);
+        v[5] = fmaf(d[0], d[2], v[5]);
+        v[6] = fmaf(d[1], d[1], v[6]);
+        v[7] = fmaf(d[1], d[2], v[7]);
+        v[8] = fmaf(d[2], d[2], v[8]);
+    }
+    fold(v, 9, false);
+    const float ic = 1.0f / fmaxf((float)cnt, 1.0f);
+    const float xy = v[4] - v[0] * v[1] * ic, xz = v[5] - v[0] * v[2] * ic, yz = v[7] - v[1] * v[2] * ic;
+    float A[3][3] = {{v[3] - v[0] * v[0] * ic, xy, xz}, {xy, v[6] - v[1] * v[1] * ic, yz},
+                     {xz, yz, v[8] - v[2] * v[2] * ic}};
+    double ax[3][3];
+    obb_axes(A, ax);
+    float a[3][3];
+    for (int k = 0; k < 3; ++k)
+        for (int r = 0; r < 3; ++r) a[k][r] = (float)ax[k][r];
+    float e[6] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max u, max -u
+    for (int k = tid; k < cnt; k += NT) {
+        const float4 p = pts[beg + k];
+        const float d[3] = {p.x - c[0], p.y - c[1], p.z - c[2]};
+        for (int r = 0; r < 3; ++r) {
+            const float u = fmaf(a[r][2], d[2], fmaf(a[r][1], d[1], a[r][0] * d[0]));
+            e[r] = fmaxf(e[r], u);
+            e[3 + r] = fmaxf(e[3 + r], -u);
+        }
+    }
+    fold(e, 6, true);
+    if (cnt > 0) {   // the middle of the extents
+        const float m[3] = {0.5f * (e[0] - e[3]), 0.5f * (e[1] - e[4]), 0.5f * (e[2] - e[5])};
+        for (int r = 0; r < 3; ++r) c[r] += fmaf(m[2], a[2][r], fmaf(m[1], a[1][r], m[0] * a[0][r]));
+    }
+    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // half-extents and radius^2 about the float centre
+    for (int k = tid; k < cnt; k += NT) {
+        const float4 p = pts[beg + k];
+        const float d[3] = {p.x - c[0], p.y - c[1], p.z - c[2]};
+        for (int r = 0; r < 3; ++r) h[r] = fmaxf(h[r], fabsf(fmaf(a[r][2], d[2], fmaf(a[r][1], d[1], a[r][0] * d[0]))));
+        h[3] = fmaxf(h[3], fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0])));
+    }
+    fold(h, 4, true);
+    if (!in || tid != 0) return;
+    if (cnt == 0) {
+        empty_obb(o);
+        return;
+    }
+    const float r = sqrtf(h[3]) * (1.0f + 1e-6f);
+    for (int k = 0; k < 3; ++k) h[k] = f32_round_up(h[k] * (1.0 + 2e-6) + 4e-6 * r + 1e-37);
+    o[0] = make_float4(c[0], c[1], c[2], h[0]);
+    for (int k = 0; k < 3; ++k) o[8 + 8 * k] = make_float4(a[k][0], a[k][1], a[k][2], k == 0 ? h[1] : (k == 1 ? h[2] : r));
+}
+
+// The levels above (few, large nodes): the axis-aligned box in the same form.
+// The first level also fills the empty positions before it (`pad`).
+__global__ void k_level_obb(const float4 *__restrict__ nodes, int L, int size, int pad, float4 *__restrict__ obb) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l < pad) empty_obb(obb_at(obb, l));
+    if (l >= size) return;
+    const int node = size + l;
+    float4 *o = obb_at(obb, wide_pos(wide_first(L), size) + l);
+    const float4 lo = nodes[2 * node], hi = nodes[2 * node + 1];
+    if (!(lo.x <= hi.x)) {
+        empty_obb(o);
+        return;
+    }
+    const float c[3] = {0.5f * lo.x + 0.5f * hi.x, 0.5f * lo.y + 0.5f * hi.y, 0.5f * lo.z + 0.5f * hi.z};
+    const float l3[3] = {lo.x, lo.y, lo.z}, h3[3] = {hi.x, hi.y, hi.z};
+    float h[3];
+    double r2 = 0.0;
+    for (int k = 0; k < 3; ++k) {
+        const double e = fmax((double)h3[k] - c[k], (double)c[k] - l3[k]);
+        r2 += e * e;
+        h[k] = (float)e;
+    }
+    const double r = sqrt(r2);
+    for (int k = 0; k < 3; ++k) h[k] = f32_round_up((double)h[k] * (1.0 + 1e-6) + 2e-6 * r + 1e-37);
+    o[0] = make_float4(c[0], c[1], c[2], h[0]);
+    o[8] = make_float4(1.0f, 0.0f, 0.0f, h[1]);
+    o[16] = make_float4(0.0f, 1.0f, 0.0f, h[2]);
+    o[24] = make_float4(0.0f, 0.0f, 1.0f, f32_round_up(r));
 }
 
 __global__ void k_level_boxes(float4 *__restrict__ nodes, int first, int count) {
@@ -340,8 +478,7 @@ __device__ bool warp_knn6(const Index &ix, int i, const float xq[3], Best6 &b, i
             } else {
                 leaf_ok = box_d2(__ldg(ix.nodes + 2 * node), __ldg(ix.nodes + 2 * node + 1), xq, zero) * kShrink
                               <= b.bound &&
-                          (ix.obb == nullptr ||
-                           obb_d2(ix.obb + 4 * (node - ix.L), xq, zero) * kObbShrink <= b.bound);
+                          obb_d2(obb_at(ix.obb, node - ix.L + ix.leaf0), xq, zero) * kObbShrink <= b.bound;
             }
         }
         int base = sp;
@@ -556,7 +693,7 @@ __device__ bool tile_knn6(const Index &ix, int g, int i, bool live, const float 
         bool need = false;
         if (live)
             need = box_d2(__ldg(ix.nodes + 2 * c), __ldg(ix.nodes + 2 * c + 1), xq, zero) * kShrink <= b.bound &&
-                   (ix.obb == nullptr || obb_d2(ix.obb + 4 * (c - ix.L), xq, zero) * kObbShrink <= b.bound);
+                   obb_d2(obb_at(ix.obb, c - ix.L + ix.leaf0), xq, zero) * kObbShrink <= b.bound;
         if (!__any_sync(FULL, need)) continue;
         const int beg = (c - ix.L) * kLeaf;
         const int end = min(beg + kLeaf, ix.n);
@@ -734,8 +871,7 @@ __device__ bool warp_knn_k(const Index &ix, int i, const float xq[3], int K, Top
             } else {
                 leaf_ok = box_d2(__ldg(ix.nodes + 2 * node), __ldg(ix.nodes + 2 * node + 1), xq, zero) * kShrink
                               <= t.bound &&
-                          (ix.obb == nullptr ||
-                           obb_d2(ix.obb + 4 * (node - ix.L), xq, zero) * kObbShrink <= t.bound);
+                          obb_d2(obb_at(ix.obb, node - ix.L + ix.leaf0), xq, zero) * kObbShrink <= t.bound;
             }
         }
         int base = sp;
@@ -1079,7 +1215,7 @@ cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cuda
     if (e != cudaSuccess) return e;
     e = cudaMalloc(&t->pts, sizeof(float4) * n);
     if (e == cudaSuccess && n_dev) e = cudaMalloc(&t->nrm, sizeof(float4) * n);
-    if (e == cudaSuccess) e = cudaMalloc(&t->nodes, sizeof(float4) * 8 * (size_t)L);
+    if (e == cudaSuccess) e = cudaMalloc(&t->nodes, sizeof(float4) * 4 * ((size_t)L + ((wide_leaf(L) + L + 7) / 8) * 8));
     if (e == cudaSuccess) {
         t->obb = t->nodes + 4 * (size_t)L;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q_dev, n_dev, order, n, t->pts, t->nrm);
@@ -1088,6 +1224,21 @@ cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cuda
         counters().launches += 3;
         for (int first = L / 2; first >= 1; first /= 2) {
             k_level_boxes<<<(first + 255) / 256, 256, 0, s>>>(t->nodes, first, first);
+            counters().launches += 1;
+        }
+        const int first = wide_first(L);
+        for (int shift = 3; (L >> shift) >= first; shift += 3) {
+            const int size = L >> shift;
+            if (shift == 3)
+                k_patch_obb<32><<<(size + 7) / 8, 256, 0, s>>>(t->pts, n, L, shift, t->nodes, t->obb);
+            else if (shift <= 9)
+                k_patch_obb<256><<<size, 256, 0, s>>>(t->pts, n, L, shift, t->nodes, t->obb);
+            else
+                k_level_obb<<<(size + 127) / 128, 128, 0, s>>>(t->nodes, L, size, 0, t->obb);
+            counters().launches += 1;
+        }
+        if (first < 8) {
+            k_level_obb<<<1, 32, 0, s>>>(t->nodes, L, 0, 8 - first, t->obb);
             counters().launches += 1;
         }
         e = cudaGetLastError();

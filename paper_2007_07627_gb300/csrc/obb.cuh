@@ -67,32 +67,13 @@ FRICP_HD inline void jacobi3f(float A[3][3], float V[3][3]) {
     }
 }
 
-// Oriented box of the cnt >= 1 points p[0 .. cnt) (.w unused), written as
-// out[0 .. 3] = (c, h0) (a0, h1) (a1, h2) (a2, r): axes along the points'
-// principal directions, made orthonormal in FP64 and rounded to float (those
-// float axes are what the box is exact for; a set that is not orthonormal to
-// 1e-6 falls back to the coordinate axes); the points' extents along them in
-// FP64 about a float centre c; the half-extents h widened by 1e-6 relative, 2e-6
-// of the radius r and 1e-12 of the coordinates' magnitude, then rounded up to
-// float.
-FRICP_HD inline void obb_fit(const float4 *p, int cnt, float4 out[4]) {
-    double s[3] = {0.0, 0.0, 0.0};
-    for (int j = 0; j < cnt; ++j) {
-        s[0] += p[j].x;
-        s[1] += p[j].y;
-        s[2] += p[j].z;
-    }
-    const float c0[3] = {(float)(s[0] / cnt), (float)(s[1] / cnt), (float)(s[2] / cnt)};
-    float A[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-    for (int j = 0; j < cnt; ++j) {
-        const float d[3] = {p[j].x - c0[0], p[j].y - c0[1], p[j].z - c0[2]};
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) A[a][b] = fmaf(d[a], d[b], A[a][b]);
-    }
+// Axes of an oriented box from the scatter matrix A (destroyed) of its points:
+// their principal directions, made orthonormal in FP64 and rounded to float (the
+// coordinate axes when that set is not orthonormal to 1e-6).
+FRICP_HD inline void obb_axes(float A[3][3], double ax[3][3]) {
     float V[3][3];
     jacobi3f(A, V);
     // Gram-Schmidt in FP64 on the first two eigenvectors, third = cross product
-    double ax[3][3];
     {
         double v0[3] = {V[0][0], V[1][0], V[2][0]}, v1[3] = {V[0][1], V[1][1], V[2][1]};
         const double n0 = sqrt(v0[0] * v0[0] + v0[1] * v0[1] + v0[2] * v0[2]);
@@ -118,6 +99,32 @@ FRICP_HD inline void obb_fit(const float4 *p, int cnt, float4 out[4]) {
     if (!ortho)
         for (int a = 0; a < 3; ++a)
             for (int b = 0; b < 3; ++b) ax[a][b] = a == b ? 1.0 : 0.0;
+}
+
+// Oriented box of the cnt >= 1 points p[0 .. cnt) (.w unused), written as
+// out[0 .. 3] = (c, h0) (a0, h1) (a1, h2) (a2, r): axes along the points'
+// principal directions, made orthonormal in FP64 and rounded to float (those
+// float axes are what the box is exact for; a set that is not orthonormal to
+// 1e-6 falls back to the coordinate axes); the points' extents along them in
+// FP64 about a float centre c; the half-extents h widened by 1e-6 relative, 2e-6
+// of the radius r and 1e-12 of the coordinates' magnitude, then rounded up to
+// float.
+FRICP_HD inline void obb_fit(const float4 *p, int cnt, float4 out[4]) {
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int j = 0; j < cnt; ++j) {
+        s[0] += p[j].x;
+        s[1] += p[j].y;
+        s[2] += p[j].z;
+    }
+    const float c0[3] = {(float)(s[0] / cnt), (float)(s[1] / cnt), (float)(s[2] / cnt)};
+    float A[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+    for (int j = 0; j < cnt; ++j) {
+        const float d[3] = {p[j].x - c0[0], p[j].y - c0[1], p[j].z - c0[2]};
+        for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 3; ++b) A[a][b] = fmaf(d[a], d[b], A[a][b]);
+    }
+    double ax[3][3];
+    obb_axes(A, ax);
     // extents about c0, then about the float centre of the box
     double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int j = 0; j < cnt; ++j) {

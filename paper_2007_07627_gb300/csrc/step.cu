@@ -1,9 +1,9 @@
 // One device step = one correspondence pass of Alg. 1 / Alg. 2 plus the
 // decision that follows it, in two kernels:
-//   k_nn_tile double-float transform (Sec. 3, x = R p + t), warm start from the
-//            previous correspondence, exact closest target point (Eq. 3), one
-//            warp per tile of kTileQ Morton-adjacent queries (tile_nn); k_nn,
-//            one warp per query (warp_nn), is the alternative search;
+//   k_nn     double-float transform (Sec. 3, x = R p + t), warm start from the
+//            previous correspondence, exact closest target point (Eq. 3), eight
+//            lanes per query (group_nn); k_nn_tile, one warp per tile of kTileQ
+//            Morton-adjacent queries (tile_nn), is the alternative search;
 //   k_accum  residual, Welsch weight and energy term (Eq. 10, Eq. 12, Eq. 16)
 //            and each point's share of the alignment sums in FP64; each block
 //            reduces its tile into one record (fixed shared-memory tree, no
@@ -16,41 +16,43 @@ namespace fricp {
 
 namespace {
 
-// Search kernel: persistent warps walk the Morton-ordered queries; each query
-// is searched by a whole warp. Writes prev[i] = this pass's correspondence (the
-// next pass's warm start).
+constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket of a first pass
+
+// Search kernel: persistent warps take runs of Morton-adjacent queries, four
+// queries at a time (search_group). Writes prev[i] = this pass's correspondence
+// (the next pass's warm start). The first run of a warp is its own index, the
+// others come from a counter in the state, so the SMs finish together and the
+// queries in flight stay in one window of the Morton order; each query's result
+// depends only on the query. A warm pass takes four queries per ticket (runs of
+// sixteen left the last tickets running alone: 335 us against 218 us, ellipsoids,
+// M = 200,000); a first pass takes longer runs, whose queries start from the
+// result of the one before.
 template <int PREC>
 __global__ void __launch_bounds__(kBlock) k_nn(StepArgs a) {
     __shared__ StepHead h;
-    __shared__ int s_stk[kBlock / 32][kWarpStack];
+    __shared__ float2 s_stk[kBlock / kGroup][kGroupStack];
     if (threadIdx.x == 0) load_head(a.st, h);
     __syncthreads();
     if (h.done) return;
-    const int wpb = kBlock / 32;
     const bool p2p = !fricp::variant_p2pl(h.variant);
-    if (p2p && h.welsch && h.phase != PH_INIT) {
-        // Welsch cap active: queries beyond it end after a round or two while the
-        // others search their neighbourhood, so a pair of queries would wait for
-        // the harder one: one query per warp
-        int *stk = s_stk[threadIdx.x >> 5];
-        for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < h.M; i += gridDim.x * wpb) {
-            if (!search_query<PREC>(a.ix, a.src, a.prev, h, i, p2p, stk) && (threadIdx.x & 31) == 0)
-                a.st->nn_overflow = 1;   // search-stack overflow: never expected
+    const int lane = threadIdx.x & 31;
+    float2 *stk = s_stk[threadIdx.x / kGroup];
+    const unsigned warps = gridDim.x * (kBlock / 32);
+    const bool cold = a.st->device_steps == 0;
+    const int rounds = cold ? max(1, min(kColdRounds, (int)(h.M / (2 * kGroupQ * warps)))) : 1;
+    unsigned e = blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+    for (;;) {
+        const long long i0 = (long long)e * (kGroupQ * rounds);
+        if (i0 >= h.M) break;
+        unsigned nx = 0;
+        if (lane == 0) nx = warps + atomicAdd(&a.st->nn_next, 1u);
+        int seed = -1;
+        for (int r = 0; r < rounds; ++r) {
+            const int i = (int)i0 + r * kGroupQ + lane / kGroup;
+            if (i - lane / kGroup >= h.M) break;
+            seed = search_group<PREC>(a.ix, a.src, a.prev, h, i, i < h.M, p2p, stk, seed);
         }
-    } else {
-        // similar work per query: two Morton-adjacent queries per warp, one per
-        // half; each warp takes the next pair from a counter in the state, so
-        // the SMs finish together (each pair's result depends only on the pair)
-        int *stk = s_stk[threadIdx.x >> 5] + (threadIdx.x & 16 ? kHalfStack : 0);
-        for (;;) {
-            unsigned e = 0;
-            if ((threadIdx.x & 31) == 0) e = atomicAdd(&a.st->nn_next, 1u);
-            e = __shfl_sync(0xffffffffu, e, 0);
-            if (2 * (long long)e >= h.M) break;
-            const int i = 2 * (int)e + ((threadIdx.x & 16) ? 1 : 0);
-            if (!search_pair<PREC>(a.ix, a.src, a.prev, h, i, i < h.M, p2p, stk) && (threadIdx.x & 31) == 0)
-                a.st->nn_overflow = 1;   // search-stack overflow: never expected
-        }
+        e = __shfl_sync(0xffffffffu, nx, 0);
     }
 }
 
@@ -97,23 +99,31 @@ __global__ void __launch_bounds__(kBlock, 3) k_accum(StepArgs a) {
         finish_pass<K>(h, a.st, a.partial, gridDim.x, a.resid, a.trace, sS, red);
 }
 
-// Correspondence step alone: index (original order) and FP64 squared distance.
-__global__ void __launch_bounds__(128) k_closest(Index ix, const float *__restrict__ p, int64_t m,
-                                                 const double *__restrict__ T, int64_t *__restrict__ idx,
-                                                 double *__restrict__ d2) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = i < m;
-    if (active) {
-        float Rh[9], Rl[9], th[3], tl[3], xh[3], xl[3];
+// Correspondence step alone: index (original order) and FP64 squared distance,
+// eight lanes per cold query. Against one thread per query the serial chain of
+// dependent loads is a fifth as long (M = N = 2,000: 114 -> 25 us) and the boxes
+// are read in whole lines (M = 80,000, N = 100,000: 1.42 -> 0.21 ms).
+__global__ void __launch_bounds__(kBlock) k_closest(Index ix, const float *__restrict__ p, int64_t m,
+                                                    const double *__restrict__ T, int64_t *__restrict__ idx,
+                                                    double *__restrict__ d2) {
+    __shared__ float2 s_stk[kBlock / kGroup][kGroupStack];
+    const int64_t i = ((int64_t)blockIdx.x * kBlock + threadIdx.x) / kGroup;
+    const bool live = i < m;
+    float xh[3] = {0.0f, 0.0f, 0.0f}, xl[3] = {0.0f, 0.0f, 0.0f};
+    float4 pp = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (live) {
+        float Rh[9], Rl[9], th[3], tl[3];
         for (int k = 0; k < 9; ++k) split_double(T[k], Rh[k], Rl[k]);
         for (int r = 0; r < 3; ++r) split_double(T[9 + r], th[r], tl[r]);
-        const float4 pp = make_float4(p[3 * i], p[3 * i + 1], p[3 * i + 2], 0.0f);
+        pp = make_float4(p[3 * i], p[3 * i + 1], p[3 * i + 2], 0.0f);
         df_transform(Rh, Rl, th, tl, pp, xh, xl);
-        NNLane q;
-        nn_init(q, xh, xl);
-        nn_thread(ix, q);
-        if (q.best_j < 0) q.best_j = 0;   // only for a non-finite x
-        const float4 qq = __ldg(ix.pts + q.best_j);
+    }
+    // a non-finite x has no closest point: position 0, as a search that accepts nothing
+    const bool finite = isfinite(xh[0] + xh[1] + xh[2]);
+    const int j = group_nn<PREC_FP64>(ix, xh, xl, __int_as_float(0x7f800000), s_stk[threadIdx.x / kGroup],
+                                      live && finite);
+    if (live && (threadIdx.x & (kGroup - 1)) == 0) {
+        const float4 qq = __ldg(ix.pts + max(j, 0));
         double x[3];
         for (int r = 0; r < 3; ++r) x[r] = fma(T[3 * r], (double)pp.x, fma(T[3 * r + 1], (double)pp.y, fma(T[3 * r + 2], (double)pp.z, T[9 + r])));
         const double dx = x[0] - (double)qq.x, dy = x[1] - (double)qq.y, dz = x[2] - (double)qq.z;
@@ -171,7 +181,7 @@ template <int PREC>
 void launch_step_prec(const StepArgs &a, int variant, int ntiles, int search, cudaStream_t s, cudaEvent_t mid) {
     static int nb_query = 0, nb_tile = 0;
     if (search == FRICP_SEARCH_QUERY)
-        k_nn<PREC><<<persistent_blocks(k_nn<PREC>, &nb_query, ntiles * kBlock, 1), kBlock, 0, s>>>(a);
+        k_nn<PREC><<<persistent_blocks(k_nn<PREC>, &nb_query, ntiles * kBlock, kGroupQ), kBlock, 0, s>>>(a);
     else
         k_nn_tile<PREC><<<persistent_blocks(k_nn_tile<PREC>, &nb_tile, ntiles * kBlock, kTileQ), kBlock, 0, s>>>(a);
     if (mid) cudaEventRecord(mid, s);
@@ -202,7 +212,8 @@ cudaError_t launch_closest(const TargetDev *t, const float *p_dev, int64_t m, co
     counters().h2d += 12 * sizeof(double);
     if (e == cudaSuccess) {
         const Index ix = make_index(*t);
-        k_closest<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(ix, p_dev, m, dT, idx, d2);
+        const int64_t per_block = kBlock / kGroup;
+        k_closest<<<(unsigned)((m + per_block - 1) / per_block), kBlock, 0, s>>>(ix, p_dev, m, dT, idx, d2);
         counters().launches += 1;
         e = cudaGetLastError();
     }

@@ -116,16 +116,9 @@ __device__ __forceinline__ void transform_point(const StepHead &h, float4 p, dou
         x[r] = fma(h.R[3 * r], (double)p.x, fma(h.R[3 * r + 1], (double)p.y, fma(h.R[3 * r + 2], (double)p.z, h.t[r])));
 }
 
-// Start a query: double-float transform, warm start from the previous
-// correspondence, and (Welsch point-to-point after the nu_max pass) the exact
-// weight cap: a point farther than the cap has weight exp(-a) = 0.0 and
-// psi = 1.0 exactly for every candidate that far, so the search radius is capped
-// there (the sums are bit-identical).
+// x = R p + t of a query as a float pair.
 template <int PREC>
-__device__ __forceinline__ void start_query(const Index &ix, const float4 *src, const int *prev, const StepHead &h,
-                                            int i, bool p2p, NNLane &q) {
-    float xh[3], xl[3];
-    const float4 p = __ldg(src + i);
+__device__ __forceinline__ void transform_query(const StepHead &h, float4 p, float xh[3], float xl[3]) {
     if (PREC == PREC_FP64) {
         df_transform(h.Rh, h.Rl, h.th, h.tl, p, xh, xl);
     } else {   // float transform with R and t rounded to float
@@ -135,10 +128,48 @@ __device__ __forceinline__ void start_query(const Index &ix, const float4 *src, 
             xl[r] = 0.0f;
         }
     }
+}
+
+// Start a query: double-float transform, warm start from the previous
+// correspondence, and (Welsch point-to-point after the nu_max pass) the exact
+// weight cap: a point farther than the cap has weight exp(-a) = 0.0 and
+// psi = 1.0 exactly for every candidate that far, so the search radius is capped
+// there (the sums are bit-identical).
+template <int PREC>
+__device__ __forceinline__ void start_query(const Index &ix, const float4 *src, const int *prev, const StepHead &h,
+                                            int i, bool p2p, NNLane &q) {
+    float xh[3], xl[3];
+    transform_query<PREC>(h, __ldg(src + i), xh, xl);
     nn_init(q, xh, xl);
     const int j0 = prev[i];
     if (j0 >= 0) nn_seed<PREC>(q, target_point<PREC>(ix, j0), j0);
     if (p2p && h.welsch && h.phase != PH_INIT && h.cut2 < q.bestf) q.bestf = h.cut2;
+}
+
+// kGroupQ queries per warp (group_nn): the lanes of a group search query i (when
+// `live`); its first lane stores the correspondence (the next pass's warm
+// start). The search is bounded by the distance to the previous correspondence,
+// or, for a query without one, to `seed` (the group's last result: the queries
+// come in Morton order, so it is near; -1: none), and by the Welsch cap
+// (start_query). Returns the correspondence.
+template <int PREC>
+__device__ __forceinline__ int search_group(const Index &ix, const float4 *src, int *prev, const StepHead &h, int i,
+                                            bool live, bool p2p, float2 *stk, int seed) {
+    float xh[3] = {0.0f, 0.0f, 0.0f}, xl[3] = {0.0f, 0.0f, 0.0f};
+    float bound = __int_as_float(0x7f800000);
+    int j0 = -1;
+    if (live) {
+        transform_query<PREC>(h, __ldg(src + i), xh, xl);
+        j0 = prev[i];
+        if (j0 < 0) j0 = seed;
+        if (j0 >= 0) bound = point_d2f(xh, xl, target_point<PREC>(ix, j0));
+        if (p2p && h.welsch && h.phase != PH_INIT) bound = fminf(bound, h.cut2);
+    }
+    int j = group_nn<PREC>(ix, xh, xl, bound, stk, live);
+    if (j < 0) j = j0 < 0 ? 0 : j0;   // nothing inside the cap
+    if (live && (threadIdx.x & (kGroup - 1)) == 0) prev[i] = j;
+    __syncwarp();
+    return live ? j : seed;
 }
 
 // One query searched by the whole warp; lane 0 stores the correspondence (the
