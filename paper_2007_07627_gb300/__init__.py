@@ -347,7 +347,7 @@ def batch_register(targets, sources, params=None, T0=None, stream=None, trace_ca
 
 def batch_set_shape(chunk: int = 0, search_blocks_per_sm: int = 1, static_order=0) -> None:
     """fricp_batch_set_shape: fix the batched launch shape (chunk = 0: autotune again).
-    static_order: 0 counter, 1 fixed stride (True), 2 query tiles."""
+    static_order: 0 counter, 1 fixed stride (True), 2 counter with chunk 8."""
     _check(lib().fricp_batch_set_shape(chunk, search_blocks_per_sm, int(static_order)))
 
 

@@ -62,7 +62,7 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
         const int64_t before = counters().launches;   // capture records launches, it does not run them
         e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            for (int k = 0; k < chunk; ++k) fricp::launch_step(a, variant, prec, ntiles, s, nullptr, prm.search);
+            for (int k = 0; k < chunk; ++k) fricp::launch_step(a, variant, prec, ntiles, s);
             e = cudaStreamEndCapture(s, &graph.g);
         }
         counters().launches = before;
@@ -84,7 +84,7 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
             if (timing)
                 for (auto &ev : iev) cudaEventCreate(&ev);
             if (timing) cudaEventRecord(iev[0], s);
-            e = fricp::launch_step(a, variant, prec, ntiles, s, timing ? iev[1] : nullptr, prm.search);
+            e = fricp::launch_step(a, variant, prec, ntiles, s, timing ? iev[1] : nullptr);
             if (timing) cudaEventRecord(iev[2], s);
             if (e == cudaSuccess) e = fricp::launch_median(a.resid, (int)init_m, mscr.p, med, s);
             if (e == cudaSuccess) e = fricp::launch_after_init(a.st, med, s);
@@ -108,7 +108,7 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
         } else {
             for (int k = 0; k < chunk && e == cudaSuccess; ++k) {
                 if (timing) cudaEventRecord(tev[3 * k], s);
-                e = fricp::launch_step(a, variant, prec, ntiles, s, timing ? tev[3 * k + 1] : nullptr, prm.search);
+                e = fricp::launch_step(a, variant, prec, ntiles, s, timing ? tev[3 * k + 1] : nullptr);
                 if (timing) cudaEventRecord(tev[3 * k + 2], s);
             }
         }
@@ -513,13 +513,12 @@ fricp_status fricp_eval_pass(const fricp_target *t, const float *p_xyz, int64_t 
     a.partial = partial.p;
     a.resid = nullptr;
     a.trace = nullptr;
-    if (e == cudaSuccess) e = fricp::launch_step(a, variant, fricp::PREC_FP64, ntiles, s, nullptr, FRICP_SEARCH_QUERY);   // a cold pass
+    if (e == cudaSuccess) e = fricp::launch_step(a, variant, fricp::PREC_FP64, ntiles, s);   // a cold pass
     PairState r;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&r, st_dev.p, sizeof(r), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "evaluation pass");
     for (int i = 0; i < 48; ++i) out[i] = r.eval_out[i];
-    if (r.nn_overflow) return fail(FRICP_EOVERFLOW, "closest-point search stack overflow");
     if (r.status == FRICP_EDEGENERATE) return fail(FRICP_EDEGENERATE, "degenerate alignment problem");
     return FRICP_OK;
 }

@@ -7,9 +7,8 @@
 //                  list, from an atomic counter (uneven registrations share
 //                  the GPU evenly) or dealt in a fixed stride (no atomics, the
 //                  warps in flight on one window of the list), whichever the
-//                  autotuner timed faster; each query is searched by a warp,
-//                  or each ticket of kTileQ queries by a warp as one query
-//                  tile (search_tile);
+//                  autotuner timed faster; a warp searches kGroupQ queries
+//                  of its ticket at a time (search_group);
 //   k_accum_batch  persistent blocks take tiles from a second counter; the
 //                  block that completes a registration's pass reduces its tile
 //                  records and runs its solver step on one warp, so the
@@ -59,8 +58,10 @@ struct BatchCtl {
 
 constexpr int kPlanThreads = 1024;
 // Order of the search tickets (BatchShape::order): from an atomic counter, in a
-// fixed stride, or query tiles of kTileQ from the counter.
+// fixed stride, or (fricp_batch_set_shape's order 2) tiles of eight queries from
+// the counter.
 constexpr int kOrderCounter = 0, kOrderStride = 1, kOrderTiles = 2;
+constexpr int kTileQ = 8;
 constexpr int kMaxSlots = 4096;
 constexpr int kSlotsPerThread = kMaxSlots / kPlanThreads;
 
@@ -148,15 +149,12 @@ __global__ void __launch_bounds__(kBlock, 4) k_nn_batch(const Slot *__restrict__
                                                      const int *__restrict__ tile_slot,
                                                      const int *__restrict__ tile_local, BatchCtl *ctl, int chunk,
                                                      unsigned max_tickets, int order) {
-    __shared__ int s_stk[kBlock / 32][kWarpStack];
-    __shared__ __align__(16) float4 s_stage[kBlock / 32][kRing * 32];
+    __shared__ float2 s_stk[kBlock / kGroup][kGroupStack];
     __shared__ StepHead s_head[kBlock / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int *stk = s_stk[w];
+    float2 *stk = s_stk[threadIdx.x / kGroup];
     StepHead &h = s_head[w];
-    const bool tiles = order == kOrderTiles;
     const int static_order = order == kOrderStride;
-    if (tiles) chunk = kTileQ;
     const int per_tile = kBlock / chunk;
     const unsigned total = min((unsigned)__ldcg(&ctl->n_tiles) * (unsigned)per_tile, max_tickets);
     int cur = -1;
@@ -184,40 +182,16 @@ __global__ void __launch_bounds__(kBlock, 4) k_nn_batch(const Slot *__restrict__
         const int i0 = lt * kBlock + sub * chunk;
         const int i1 = min(i0 + chunk, h.M);
         const bool p2p = !fricp::variant_p2pl(h.variant);
-        if (tiles) {   // the ticket's queries as one query tile
-            bool ok;
+        int seed = -1;
+        for (int k = i0; k < i1; k += kGroupQ) {
+            const int i = k + lane / kGroup;
+            const bool live = i < i1;
             if (h.prec == PREC_FP32)
-                ok = search_tile<PREC_FP32>(sl.ix, sl.src, sl.prev, h, i0, i1, p2p, stk, s_stage[w]);
+                seed = search_group<PREC_FP32>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed);
             else if (h.prec == PREC_FP16)
-                ok = search_tile<PREC_FP16>(sl.ix, sl.src, sl.prev, h, i0, i1, p2p, stk, s_stage[w]);
+                seed = search_group<PREC_FP16>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed);
             else
-                ok = search_tile<PREC_FP64>(sl.ix, sl.src, sl.prev, h, i0, i1, p2p, stk, s_stage[w]);
-            if (!ok && lane == 0) sl.st->nn_overflow = 1;   // search-stack overflow: never expected
-        } else if (p2p && h.welsch && h.phase != PH_INIT) {   // Welsch cap active: one query per warp (as k_nn)
-            for (int i = i0; i < i1; ++i) {
-                bool ok;
-                if (h.prec == PREC_FP32)
-                    ok = search_query<PREC_FP32>(sl.ix, sl.src, sl.prev, h, i, p2p, stk);
-                else if (h.prec == PREC_FP16)
-                    ok = search_query<PREC_FP16>(sl.ix, sl.src, sl.prev, h, i, p2p, stk);
-                else
-                    ok = search_query<PREC_FP64>(sl.ix, sl.src, sl.prev, h, i, p2p, stk);
-                if (!ok && lane == 0) sl.st->nn_overflow = 1;   // search-stack overflow: never expected
-            }
-        } else {   // two queries per warp, one per half
-            int *hstk = stk + ((lane & 16) ? kHalfStack : 0);
-            for (int i2 = i0; i2 < i1; i2 += 2) {
-                const int i = i2 + ((lane & 16) ? 1 : 0);
-                const bool live = i < i1;
-                bool ok;
-                if (h.prec == PREC_FP32)
-                    ok = search_pair<PREC_FP32>(sl.ix, sl.src, sl.prev, h, i, live, p2p, hstk);
-                else if (h.prec == PREC_FP16)
-                    ok = search_pair<PREC_FP16>(sl.ix, sl.src, sl.prev, h, i, live, p2p, hstk);
-                else
-                    ok = search_pair<PREC_FP64>(sl.ix, sl.src, sl.prev, h, i, live, p2p, hstk);
-                if (!ok && lane == 0) sl.st->nn_overflow = 1;   // search-stack overflow: never expected
-            }
+                seed = search_group<PREC_FP64>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed);
         }
     }
 }
@@ -462,12 +436,12 @@ class BatchEngine {
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
-        // (chunk, order): query tiles, tickets of 1 or 4 queries from the counter,
-        // single queries in a fixed stride (the shapes that have won on some
-        // size class: tiles on every mix of many or large registrations, the
-        // others on a few small ones)
-        const int cands[][2] = {{kTileQ, kOrderTiles}, {4, kOrderCounter}, {1, kOrderCounter}, {1, kOrderStride}};
-        int per_sm[2] = {nn_max, (nn_max + 1) / 2};
+        // (chunk, order): tickets of one or two rounds of kGroupQ queries from
+        // the counter, one round in a fixed stride (tickets of 16 and half the
+        // blocks were never the fastest: 16 mixed pairs, M 2k-200k, 169 ms per
+        // batch with tickets of 4, 176 with 8, 194 with 16, 173 in a stride, 197
+        // with half the blocks)
+        const int cands[][2] = {{kGroupQ, kOrderCounter}, {2 * kGroupQ, kOrderCounter}, {kGroupQ, kOrderStride}};
         BatchShape best{1, nn_max, acc_max, 0};
         float best_ms = 1e30f;
         cudaError_t e = cudaSuccess;
@@ -477,22 +451,19 @@ class BatchEngine {
         counters().launches += 1;
         for (const auto &cd : cands) {
             const int c = cd[0], so = cd[1];
-            for (int pi = 0; pi < 2; ++pi) {
-                const int ps = per_sm[pi];
-                if (ps < 1 || ps > nn_max || (pi == 1 && ps == per_sm[0])) continue;
-                k_reset_nn_ticket<<<1, 1, 0, s>>>(d_ctl);
-                cudaEventRecord(e0, s);
-                k_nn_batch<<<sm_count() * ps, kBlock, 0, s>>>(d_slots, d_heads, d_tile_slot, d_tile_local, d_ctl, c,
+            k_reset_nn_ticket<<<1, 1, 0, s>>>(d_ctl);
+            cudaEventRecord(e0, s);
+            k_nn_batch<<<sm_count() * nn_max, kBlock, 0, s>>>(d_slots, d_heads, d_tile_slot, d_tile_local, d_ctl, c,
                                                               0xffffffffu, so);
-                cudaEventRecord(e1, s);
-                counters().launches += 2;
-                e = cudaEventSynchronize(e1);
-                if (e != cudaSuccess) break;
+            cudaEventRecord(e1, s);
+            counters().launches += 2;
+            e = cudaEventSynchronize(e1);
+            if (e == cudaSuccess) {
                 float ms = 0.0f;
                 cudaEventElapsedTime(&ms, e0, e1);
                 if (ms < best_ms) {
                     best_ms = ms;
-                    best = BatchShape{c, ps, acc_max, so};
+                    best = BatchShape{c, nn_max, acc_max, so};
                 }
             }
             if (e != cudaSuccess) break;

@@ -143,7 +143,7 @@ extern "C" fricp_status fricp_eval_pass_static(const fricp_target *target, const
     a.partial = partial;
     a.resid = nullptr;
     a.trace = nullptr;
-    if (e == cudaSuccess) e = fricp::launch_step(a, variant, fricp::PREC_FP64, ntiles, s, nullptr, FRICP_SEARCH_QUERY);   // a cold pass
+    if (e == cudaSuccess) e = fricp::launch_step(a, variant, fricp::PREC_FP64, ntiles, s);   // a cold pass
     PairState r;
     int bad = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&r, st_dev, sizeof(r), cudaMemcpyDeviceToHost, s);
@@ -153,7 +153,6 @@ extern "C" fricp_status fricp_eval_pass_static(const fricp_target *target, const
     fricp::counters().h2d += sizeof(h) + sizeof(T12);
     fricp::counters().d2h += sizeof(r) + sizeof(int);
     if (bad) return static_fail(FRICP_EINVAL, "p_xyz has NaN or Inf");
-    if (r.nn_overflow) return static_fail(FRICP_EOVERFLOW, "closest-point search stack overflow");
     for (int i = 0; i < 48; ++i) out[i] = r.eval_out[i];
     if (r.status == FRICP_EDEGENERATE) return static_fail(FRICP_EDEGENERATE, "degenerate alignment problem");
     return FRICP_OK;

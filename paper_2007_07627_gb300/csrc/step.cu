@@ -2,8 +2,7 @@
 // decision that follows it, in two kernels:
 //   k_nn     double-float transform (Sec. 3, x = R p + t), warm start from the
 //            previous correspondence, exact closest target point (Eq. 3), eight
-//            lanes per query (group_nn); k_nn_tile, one warp per tile of kTileQ
-//            Morton-adjacent queries (tile_nn), is the alternative search;
+//            lanes per query (group_nn);
 //   k_accum  residual, Welsch weight and energy term (Eq. 10, Eq. 12, Eq. 16)
 //            and each point's share of the alignment sums in FP64; each block
 //            reduces its tile into one record (fixed shared-memory tree, no
@@ -53,32 +52,6 @@ __global__ void __launch_bounds__(kBlock) k_nn(StepArgs a) {
             seed = search_group<PREC>(a.ix, a.src, a.prev, h, i, i < h.M, p2p, stk, seed);
         }
         e = __shfl_sync(0xffffffffu, nx, 0);
-    }
-}
-
-// Search kernel over query tiles: persistent warps take tiles of kTileQ
-// Morton-adjacent queries (four lanes per query, search_tile) from a counter
-// in the state (the tiles' costs vary with the surface and the outliers they
-// hold). Each result depends only on its query, so the order changes no bit.
-template <int PREC>
-__global__ void __launch_bounds__(kBlock) k_nn_tile(StepArgs a) {
-    __shared__ StepHead h;
-    __shared__ int s_buf[kBlock / 32][kWarpStack];
-    __shared__ __align__(16) float4 s_stage[kBlock / 32][kRing * 32];
-    if (threadIdx.x == 0) load_head(a.st, h);
-    __syncthreads();
-    if (h.done) return;
-    const bool p2p = !fricp::variant_p2pl(h.variant);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned e = 0;
-        if (lane == 0) e = atomicAdd(&a.st->nn_next, 1u);
-        e = __shfl_sync(0xffffffffu, e, 0);
-        if ((long long)kTileQ * e >= h.M) break;
-        const int i0 = kTileQ * (int)e;
-        if (!search_tile<PREC>(a.ix, a.src, a.prev, h, i0, min(i0 + kTileQ, h.M), p2p, s_buf[w], s_stage[w]) &&
-            lane == 0)
-            a.st->nn_overflow = 1;   // search-stack overflow: never expected
     }
 }
 
@@ -178,12 +151,9 @@ int persistent_blocks(K kernel, int *cache, int M, int per_warp) {
 }
 
 template <int PREC>
-void launch_step_prec(const StepArgs &a, int variant, int ntiles, int search, cudaStream_t s, cudaEvent_t mid) {
-    static int nb_query = 0, nb_tile = 0;
-    if (search == FRICP_SEARCH_QUERY)
-        k_nn<PREC><<<persistent_blocks(k_nn<PREC>, &nb_query, ntiles * kBlock, kGroupQ), kBlock, 0, s>>>(a);
-    else
-        k_nn_tile<PREC><<<persistent_blocks(k_nn_tile<PREC>, &nb_tile, ntiles * kBlock, kTileQ), kBlock, 0, s>>>(a);
+void launch_step_prec(const StepArgs &a, int variant, int ntiles, cudaStream_t s, cudaEvent_t mid) {
+    static int nb = 0;
+    k_nn<PREC><<<persistent_blocks(k_nn<PREC>, &nb, ntiles * kBlock, kGroupQ), kBlock, 0, s>>>(a);
     if (mid) cudaEventRecord(mid, s);
     if (fricp::variant_p2pl(variant))
         k_accum<1, PREC><<<ntiles, kBlock, 0, s>>>(a);
@@ -191,14 +161,13 @@ void launch_step_prec(const StepArgs &a, int variant, int ntiles, int search, cu
         k_accum<0, PREC><<<ntiles, kBlock, 0, s>>>(a);
 }
 
-cudaError_t launch_step(const StepArgs &a, int variant, int prec, int ntiles, cudaStream_t s, cudaEvent_t mid,
-                        int search) {
+cudaError_t launch_step(const StepArgs &a, int variant, int prec, int ntiles, cudaStream_t s, cudaEvent_t mid) {
     if (prec == PREC_FP32)
-        launch_step_prec<PREC_FP32>(a, variant, ntiles, search, s, mid);
+        launch_step_prec<PREC_FP32>(a, variant, ntiles, s, mid);
     else if (prec == PREC_FP16)
-        launch_step_prec<PREC_FP16>(a, variant, ntiles, search, s, mid);
+        launch_step_prec<PREC_FP16>(a, variant, ntiles, s, mid);
     else
-        launch_step_prec<PREC_FP64>(a, variant, ntiles, search, s, mid);
+        launch_step_prec<PREC_FP64>(a, variant, ntiles, s, mid);
     counters().launches += 2;
     return cudaGetLastError();
 }

@@ -130,28 +130,14 @@ __device__ __forceinline__ void transform_query(const StepHead &h, float4 p, flo
     }
 }
 
-// Start a query: double-float transform, warm start from the previous
-// correspondence, and (Welsch point-to-point after the nu_max pass) the exact
-// weight cap: a point farther than the cap has weight exp(-a) = 0.0 and
-// psi = 1.0 exactly for every candidate that far, so the search radius is capped
-// there (the sums are bit-identical).
-template <int PREC>
-__device__ __forceinline__ void start_query(const Index &ix, const float4 *src, const int *prev, const StepHead &h,
-                                            int i, bool p2p, NNLane &q) {
-    float xh[3], xl[3];
-    transform_query<PREC>(h, __ldg(src + i), xh, xl);
-    nn_init(q, xh, xl);
-    const int j0 = prev[i];
-    if (j0 >= 0) nn_seed<PREC>(q, target_point<PREC>(ix, j0), j0);
-    if (p2p && h.welsch && h.phase != PH_INIT && h.cut2 < q.bestf) q.bestf = h.cut2;
-}
-
 // kGroupQ queries per warp (group_nn): the lanes of a group search query i (when
 // `live`); its first lane stores the correspondence (the next pass's warm
 // start). The search is bounded by the distance to the previous correspondence,
 // or, for a query without one, to `seed` (the group's last result: the queries
-// come in Morton order, so it is near; -1: none), and by the Welsch cap
-// (start_query). Returns the correspondence.
+// come in Morton order, so it is near; -1: none), and, for Welsch point-to-point
+// after the nu_max pass, by the exact weight cap: a point farther than the cap
+// has weight exp(-a) = 0.0 and psi = 1.0 exactly for every candidate that far, so
+// the sums are bit-identical. Returns the correspondence.
 template <int PREC>
 __device__ __forceinline__ int search_group(const Index &ix, const float4 *src, int *prev, const StepHead &h, int i,
                                             bool live, bool p2p, float2 *stk, int seed) {
@@ -170,70 +156,6 @@ __device__ __forceinline__ int search_group(const Index &ix, const float4 *src, 
     if (live && (threadIdx.x & (kGroup - 1)) == 0) prev[i] = j;
     __syncwarp();
     return live ? j : seed;
-}
-
-// One query searched by the whole warp; lane 0 stores the correspondence (the
-// next pass's warm start). Returns false on a search-stack overflow.
-template <int PREC>
-__device__ __forceinline__ bool search_query(const Index &ix, const float4 *src, int *prev, const StepHead &h, int i,
-                                             bool p2p, int *stk) {
-    NNLane q;   // every lane sets up the same query (float arithmetic, broadcast loads)
-    start_query<PREC>(ix, src, prev, h, i, p2p, q);
-    const bool ok = warp_nn<PREC>(ix, q, stk, q.best_j >= 0 ? q.best_j / kLeaf : -1);
-    if (!ok) q.best_j = 0;
-    if ((threadIdx.x & 31) == 0) prev[i] = q.best_j < 0 ? 0 : q.best_j;   // -1 only if nothing lies inside the cap
-    __syncwarp();
-    return ok;
-}
-
-// Two queries per warp (halfwarp_nn): lanes 0-15 search query i, lanes 16-31
-// query i + 1 (when `live`); lane 0 of each half stores its correspondence.
-// Returns false on a search-stack overflow.
-template <int PREC>
-__device__ __forceinline__ bool search_pair(const Index &ix, const float4 *src, int *prev, const StepHead &h, int i,
-                                            bool live, bool p2p, int *stk_half) {
-    NNLane q;
-    if (live) {
-        start_query<PREC>(ix, src, prev, h, i, p2p, q);
-    } else {
-        const float z[3] = {0.0f, 0.0f, 0.0f};
-        nn_init(q, z, z);
-    }
-    const bool ok = halfwarp_nn<PREC>(ix, q, stk_half, live && q.best_j >= 0 ? q.best_j / kLeaf : -1, live);
-    if (live && (threadIdx.x & 15) == 0) prev[i] = (!ok || q.best_j < 0) ? 0 : q.best_j;
-    __syncwarp();
-    return ok;
-}
-
-// Queries i0 .. i0 + kTileQ - 1 (below i1) as one query tile (tile_nn); the
-// queries it sets aside (no warm start: the first pass) are then searched one
-// by one by the whole warp (warp_nn). The group head stores each
-// correspondence. `wbuf`: kWarpStack ints per warp; `stage`: kRing x 32
-// float4. Returns false on a search-stack overflow.
-template <int PREC>
-__device__ __forceinline__ bool search_tile(const Index &ix, const float4 *src, int *prev, const StepHead &h, int i0,
-                                            int i1, bool p2p, int *wbuf, float4 *stage) {
-    const int lane = threadIdx.x & 31;
-    const int i = i0 + (lane >> 2);
-    const bool live = i < i1;
-    NNLane q;
-    if (live) {
-        start_query<PREC>(ix, src, prev, h, i, p2p, q);
-    } else {
-        const float z[3] = {0.0f, 0.0f, 0.0f};
-        nn_init(q, z, z);
-    }
-    const unsigned aside = tile_nn<PREC>(ix, q, live, wbuf, wbuf + kTileStack, stage);
-    if (live && (lane & 3) == 0 && !((aside >> lane) & 1u)) prev[i] = q.best_j;   // warm-started: best_j >= 0
-    __syncwarp();
-    bool ok = true;
-    unsigned heads = aside & 0x11111111u;
-    while (heads) {
-        const int g = (__ffs(heads) - 1) >> 2;
-        heads &= heads - 1u;
-        ok = search_query<PREC>(ix, src, prev, h, i0 + g, p2p, wbuf) && ok;
-    }
-    return ok;
 }
 
 // Point i's share of the pass sums at this pass's correspondence:
