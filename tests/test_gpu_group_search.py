@@ -94,3 +94,27 @@ def test_both_search_layouts_agree(fr, n, precision):
     assert a["status"] == b["status"] and a["iterations"] == b["iterations"]
     assert np.array_equal(a["R"], b["R"]) and np.array_equal(a["t"], b["t"]) and np.array_equal(a["trace"], b["trace"])
     t.destroy()
+
+
+@pytest.mark.parametrize("m", [(1 << 17) - 1, 1 << 17, (1 << 17) + 37])
+def test_queries_dealt_by_cell(fr, m):
+    """From 2^17 queries on the search deals them by cell first: points inside and
+    far outside the target's box, duplicates and non-finite ones land at their own
+    place, with the index and distance of a small call on the same points."""
+    import torch
+    g = np.random.default_rng(m)
+    Q = np.concatenate([g.random((5000, 3)), np.repeat(g.random((1, 3)), 50, 0)]).astype(np.float32)
+    P = np.concatenate([g.random((m - 4000, 3)), 40.0 * g.standard_normal((2000, 3)),
+                        np.repeat(g.random((1, 3)), 1990, 0), np.full((10, 3), np.nan)]).astype(np.float32)
+    P = P[g.permutation(m)]
+    t, p = fr.target_create(_dev(Q)), _dev(P)
+    T = np.eye(4)
+    T[:3, 3] = (0.01, -0.02, 0.03)
+    idx, d2 = fr.closest_points(t, p, T)
+    for lo in (0, m // 2, m - 3001):
+        i1, e1 = fr.closest_points(t, p[lo:lo + 3001], T)
+        assert torch.equal(idx[lo:lo + 3001], i1) and torch.equal(d2[lo:lo + 3001].nan_to_num(-1.0), e1.nan_to_num(-1.0))
+    near = np.flatnonzero(np.isfinite(P).all(1))[:200]
+    io, _ = _brute(P[near].astype(np.float64) + T[:3, 3], Q)
+    assert np.array_equal(idx.cpu().numpy()[near], io)
+    t.destroy()
