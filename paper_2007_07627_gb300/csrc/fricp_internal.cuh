@@ -431,7 +431,8 @@ __device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], c
     const unsigned below = (1u << gl) - 1u;
     const int leaf0 = AABB ? ix.L : ix.leaf0;     // first bucket: as a node of the binary tree, or a position
     int base = AABB ? ix.first : 0;               // first of the eight boxes this round tests
-    int cnt = live ? (AABB ? ix.first : 8) : 0;   // how many of them (eight after the first round)
+    int cnt = live ? ix.first : 0;                // how many of them are nodes: eight after the first round, whose
+                                                  // positions begin with 8 - first empty boxes that must not be entered
     int sp = 0;
     while (__any_sync(FULL, cnt != 0)) {
         const bool leaf = AABB ? base >= leaf0 : base + 7 >= leaf0;
@@ -441,7 +442,7 @@ __device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], c
         for (int c = 0; c < kGroupC; ++c) {
             const int g = gl + c * kGroup;
             key[c] = OUT;
-            if (AABB ? g < cnt : cnt != 0) {
+            if (AABB ? g < cnt : g >= 8 - cnt) {
                 if (AABB)
                     key[c] = box_d2(__ldg(ix.nodes + 2 * (base + g)), __ldg(ix.nodes + 2 * (base + g) + 1), xh, xl) *
                              kShrink;

@@ -151,7 +151,9 @@ __device__ __forceinline__ int search_group(const Index &ix, const float4 *src, 
         if (j0 >= 0) bound = point_d2f(xh, xl, target_point<PREC>(ix, j0));
         if (p2p && h.welsch && h.phase != PH_INIT) bound = fminf(bound, h.cut2);
     }
-    int j = group_nn<PREC>(ix, xh, xl, bound, stk, live);
+    // (fricp_eval_pass_static also searches non-finite points, which it then rejects)
+    const bool finite = isfinite(xh[0] + xh[1] + xh[2]);
+    int j = group_nn<PREC>(ix, xh, xl, bound, stk, live && finite);
     if (j < 0) j = j0 < 0 ? 0 : j0;   // nothing inside the cap
     if (live && (threadIdx.x & (kGroup - 1)) == 0) prev[i] = j;
     __syncwarp();
