@@ -4,6 +4,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -30,6 +31,11 @@ using fricp::counters;
 using namespace fricp::host;
 
 thread_local std::string g_err;
+
+void free_target(TargetDev *t, cudaStream_t s) {
+    for (void *p : {(void *)t->pts, (void *)t->nrm, (void *)t->nodes, (void *)t->pts16})
+        if (p) cudaFreeAsync(p, s);
+}
 
 // Run fused steps until the state machine is done. Returns the status and the
 // summed device time of the step launches when timing is requested.
@@ -153,6 +159,50 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
 }  // namespace
 
 namespace fricp {
+
+// The library's memory pool on the current device. The device's default pool
+// returns its memory to the driver at every synchronisation, so each call paid
+// for mapping its buffers again (eval_pass on 2,000 points: 416 us, about 200 of
+// them in allocations); this one keeps up to kPoolKeep bytes, and gives them back
+// when an allocation does not fit. Pools are shared by all threads and streams.
+static cudaMemPool_t device_pool() {
+    constexpr int kMaxDevices = 64;
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (pools[dev] == nullptr) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof(props));
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        uint64_t keep = kPoolKeep;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        pools[dev] = pool;
+    }
+    return pools[dev];
+}
+
+cudaError_t pool_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    const cudaMemPool_t pool = device_pool();
+    if (pool == nullptr) return cudaMallocAsync(p, bytes, s);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {   // give back what is kept but unused, once
+        cudaGetLastError();
+        cudaStreamSynchronize(s);
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return e;
+}
+
 const TargetDev *target_dev(const fricp_target *t) { return t ? &t->d : nullptr; }
 void set_last_error(const char *msg) { g_err = msg; }
 }  // namespace fricp
@@ -214,9 +264,7 @@ fricp_status fricp_target_create(const float *q_xyz, const float *q_normals, int
     int bad = 0;
     cudaError_t e = fricp::build_target(q.ptr, q_normals ? nq.ptr : nullptr, n, ord.work, &t->d, &bad);
     if (e != cudaSuccess || bad) {
-        if (t->d.pts) cudaFree(t->d.pts);
-        if (t->d.nrm) cudaFree(t->d.nrm);
-        if (t->d.nodes) cudaFree(t->d.nodes);
+        free_target(&t->d, ord.work);
         delete t;
         if (bad) return fail(FRICP_EINVAL, "target has NaN/Inf coordinates or non-unit normals");
         return e == cudaErrorMemoryAllocation ? fail(FRICP_ENOMEM, "device allocation for the target index")
@@ -257,8 +305,7 @@ fricp_status fricp_estimate_normals(const float *q_xyz, int64_t n, int32_t k, in
         counters().d2h += (int64_t)sizeof(float) * 3 * n;
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }
-    if (t.pts) cudaFree(t.pts);
-    if (t.nodes) cudaFree(t.nodes);
+    free_target(&t, s);
     if (bad) return fail(FRICP_EINVAL, "q_xyz has NaN or Inf");
     if (e == cudaErrorMemoryAllocation) return fail(FRICP_ENOMEM, "device allocation for the normal estimate");
     if (e != cudaSuccess) return cuda_fail(e, "normal estimate");
@@ -269,10 +316,7 @@ fricp_status fricp_estimate_normals(const float *q_xyz, int64_t n, int32_t k, in
 fricp_status fricp_target_destroy(fricp_target *t) {
     if (t == nullptr) return FRICP_OK;
     cudaDeviceSynchronize();
-    if (t->d.pts) cudaFree(t->d.pts);
-    if (t->d.nrm) cudaFree(t->d.nrm);
-    if (t->d.nodes) cudaFree(t->d.nodes);
-    if (t->d.pts16) cudaFree(t->d.pts16);
+    free_target(&t->d, work_stream());
     delete t;
     return FRICP_OK;
 }
@@ -480,11 +524,10 @@ fricp_status fricp_eval_pass(const fricp_target *t, const float *p_xyz, int64_t 
     const int ntiles = (int)((m + fricp::kBlock - 1) / fricp::kBlock);
     DevBuf<float4> src;
     DevBuf<PairState> st_dev;
-    DevBuf<double> partial, Tdev;
+    DevBuf<double> partial;
     DevBuf<int> prev;
     if (src.alloc(m, s) != cudaSuccess || st_dev.alloc(1, s) != cudaSuccess || prev.alloc(m, s) != cudaSuccess ||
-        partial.alloc((size_t)ntiles * fricp::kMaxSums, s) != cudaSuccess ||
-        Tdev.alloc(12, s) != cudaSuccess)
+        partial.alloc((size_t)ntiles * fricp::kMaxSums, s) != cudaSuccess)
         return fail(FRICP_ENOMEM, "device allocation");
     float plo[3], phi[3];
     int bad = 0;
@@ -496,15 +539,9 @@ fricp_status fricp_eval_pass(const fricp_target *t, const float *p_xyz, int64_t 
     const double c[3] = {center ? center[0] : 0.0, center ? center[1] : 0.0, center ? center[2] : 0.0};
     PairState h = initial_state(prm, m, ntiles, scale, c, 1.0, 0);
     h.nu = fricp::variant_robust(variant) ? nu : 1.0;
-    double T12[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int k = 0; k < 3; ++k) T12[3 * r + k] = T_normalized[4 * r + k];
-        T12[9 + r] = T_normalized[4 * r + 3];
-    }
+    setup_eval(&h, T_normalized);
     e = cudaMemcpyAsync(st_dev.p, &h, sizeof(h), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(prev.p, 0xff, sizeof(int) * m, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(Tdev.p, T12, sizeof(T12), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = fricp::launch_setup_eval_xi(st_dev.p, Tdev.p, s);
     fricp::StepArgs a;
     a.st = st_dev.p;
     a.ix = fricp::make_index(t->d);

@@ -312,12 +312,12 @@ class BatchEngine {
 
     void release() {
         graph.reset();
-        if (d_slots) cudaFree(d_slots);
-        if (d_heads) cudaFree(d_heads);
-        if (d_done) cudaFree(d_done);
-        if (d_tile_slot) cudaFree(d_tile_slot);
-        if (d_tile_local) cudaFree(d_tile_local);
-        if (d_ctl) cudaFree(d_ctl);
+        if (d_slots) cudaFreeAsync(d_slots, s);
+        if (d_heads) cudaFreeAsync(d_heads, s);
+        if (d_done) cudaFreeAsync(d_done, s);
+        if (d_tile_slot) cudaFreeAsync(d_tile_slot, s);
+        if (d_tile_local) cudaFreeAsync(d_tile_local, s);
+        if (d_ctl) cudaFreeAsync(d_ctl, s);
         if (h_done) cudaFreeHost(h_done);
         if (h_ctl) cudaFreeHost(h_ctl);
         d_slots = nullptr;
@@ -332,12 +332,12 @@ class BatchEngine {
         s = stream;
         max_slots = slots;
         max_tiles = tiles > 0 ? tiles : 1;
-        cudaError_t e = cudaMalloc(&d_slots, sizeof(Slot) * slots);
-        if (e == cudaSuccess) e = cudaMalloc(&d_heads, sizeof(StepHead) * slots);
-        if (e == cudaSuccess) e = cudaMalloc(&d_done, sizeof(int) * slots);
-        if (e == cudaSuccess) e = cudaMalloc(&d_tile_slot, sizeof(int) * max_tiles);
-        if (e == cudaSuccess) e = cudaMalloc(&d_tile_local, sizeof(int) * max_tiles);
-        if (e == cudaSuccess) e = cudaMalloc(&d_ctl, sizeof(BatchCtl));
+        cudaError_t e = pool_alloc(&d_slots, sizeof(Slot) * slots, s);
+        if (e == cudaSuccess) e = pool_alloc(&d_heads, sizeof(StepHead) * slots, s);
+        if (e == cudaSuccess) e = pool_alloc(&d_done, sizeof(int) * slots, s);
+        if (e == cudaSuccess) e = pool_alloc(&d_tile_slot, sizeof(int) * max_tiles, s);
+        if (e == cudaSuccess) e = pool_alloc(&d_tile_local, sizeof(int) * max_tiles, s);
+        if (e == cudaSuccess) e = pool_alloc(&d_ctl, sizeof(BatchCtl), s);
         if (e == cudaSuccess) e = cudaMallocHost(&h_done, sizeof(int) * slots);
         if (e == cudaSuccess) e = cudaMallocHost(&h_ctl, sizeof(BatchCtl));
         if (e == cudaSuccess) e = cudaMemsetAsync(d_slots, 0, sizeof(Slot) * slots, s);
@@ -509,7 +509,7 @@ struct PairBuffers {
     }
     cudaError_t alloc(int64_t m, int trace_cap, cudaStream_t s) {
         bytes = need(m, trace_cap);
-        cudaError_t e = cudaMallocAsync(&base, bytes, s);
+        cudaError_t e = fricp::pool_alloc(&base, bytes, s);
         if (e != cudaSuccess) return e;
         const int64_t ntiles = (m + fricp::kBlock - 1) / fricp::kBlock;
         char *p = base;
@@ -949,7 +949,7 @@ extern "C" fricp_status fricp_server_submit(fricp_server *sv, const fricp_target
     if (on_device) {
         cudaError_t e = cudaEventRecord(sv->ev_user, sv->user);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(sv->s_admit, sv->ev_user, 0);
-        if (e == cudaSuccess) e = cudaMallocAsync(&r.dev_pts, sizeof(float) * 3 * m, sv->s_admit);
+        if (e == cudaSuccess) e = fricp::pool_alloc(&r.dev_pts, sizeof(float) * 3 * m, sv->s_admit);
         if (e != cudaSuccess) return fail(FRICP_ENOMEM, "device copy of a request");
         e = cudaMemcpyAsync(r.dev_pts, p_xyz, sizeof(float) * 3 * m, cudaMemcpyDeviceToDevice, sv->s_admit);
         if (e == cudaSuccess) e = cudaEventRecord(sv->ev_user, sv->s_admit);

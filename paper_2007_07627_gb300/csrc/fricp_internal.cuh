@@ -609,6 +609,15 @@ Counters &counters();
 const TargetDev *target_dev(const fricp_target *t);
 void set_last_error(const char *msg);
 
+// Stream-ordered device memory from the library's own pool (api.cu). Freed with
+// cudaFreeAsync; the pool keeps up to kPoolKeep bytes across synchronisations.
+constexpr size_t kPoolKeep = (size_t)256 << 20;
+cudaError_t pool_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
+template <class T>
+inline cudaError_t pool_alloc(T **p, size_t bytes, cudaStream_t s) {
+    return pool_alloc_bytes(reinterpret_cast<void **>(p), bytes, s);
+}
+
 cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cudaStream_t s,
                          TargetDev *t, int *bad_input);
 cudaError_t target_nu_stats(TargetDev *t, cudaStream_t s);
@@ -627,7 +636,6 @@ cudaError_t launch_closest(const TargetDev *t, const float *p_dev, int64_t m, co
 // kernel. When `mid` is given it is recorded between the two.
 cudaError_t launch_step(const StepArgs &a, int variant, int prec, int ntiles, cudaStream_t s,
                         cudaEvent_t mid = nullptr);
-cudaError_t launch_setup_eval_xi(PairState *st, const double *T_normalized12, cudaStream_t s);
 // Median of n non-negative doubles (the mean of the two middle order
 // statistics, exact) by a grid-wide 8-bit radix select; `scratch` holds
 // kMedianScratchBytes of device memory, the result lands in *out_dev.

@@ -97,7 +97,7 @@ inline fricp_status stage_input(const float *x, int64_t n, int on_device, cudaSt
         return FRICP_OK;
     }
     if (!host_finite(x, 3 * n)) return fail(FRICP_EINVAL, std::string(what) + " has NaN or Inf");
-    cudaError_t e = cudaMallocAsync(&out->owned, sizeof(float) * 3 * n, s);
+    cudaError_t e = pool_alloc(&out->owned, sizeof(float) * 3 * n, s);
     if (e != cudaSuccess) return fail(FRICP_ENOMEM, std::string("device allocation for ") + what);
     e = cudaMemcpyAsync(out->owned, x, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "copy input to device");
@@ -113,7 +113,7 @@ struct DevBuf {
     bool leak = false;
     cudaError_t alloc(size_t count, cudaStream_t st) {
         s = st;
-        return cudaMallocAsync(&p, sizeof(T) * (count > 0 ? count : 1), st);
+        return pool_alloc(&p, sizeof(T) * (count > 0 ? count : 1), st);
     }
     ~DevBuf() {
         if (p && !leak) cudaFreeAsync(p, s);
@@ -268,6 +268,26 @@ inline fricp_status setup_pair(const TargetDev &t, const fricp_params &prm, int6
     }
     set_head_cache_serial(h);
     return FRICP_OK;
+}
+
+// A single evaluation at a normalised transform (double[16], row-major) for
+// fricp_eval_pass: the state its one pass starts from.
+inline void setup_eval(PairState *h, const double *T_normalized) {
+    double Tn[12], xi[6];
+    for (int r = 0; r < 3; ++r) {
+        for (int k = 0; k < 3; ++k) Tn[3 * r + k] = T_normalized[4 * r + k];
+        Tn[9 + r] = T_normalized[4 * r + 3];
+    }
+    std::vector<double> sh(kTeamScratch);
+    const Team tm{sh.data()};
+    if (fricp::variant_p2pl(h->variant)) {
+        log_state_T(tm, Tn, xi);
+        request_eval_xi(tm, h, xi, 1);
+    } else {
+        request_eval_state_T(tm, h, Tn, 1);
+    }
+    h->phase = PH_EVAL;
+    set_head_cache_serial(h);
 }
 
 // Caller-facing result from a registration's final state.

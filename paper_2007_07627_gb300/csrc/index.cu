@@ -1109,7 +1109,7 @@ cudaError_t reduce_box(const float *x, const float *nrm, int64_t n, cudaStream_t
     int nb = (int)std::min<int64_t>((n + kRedBlock - 1) / kRedBlock, 1024);
     if (nb < 1) nb = 1;
     BoxPartial *parts = nullptr;
-    cudaError_t e = cudaMallocAsync(&parts, sizeof(BoxPartial) * (nb + 1), s);
+    cudaError_t e = pool_alloc(&parts, sizeof(BoxPartial) * (nb + 1), s);
     if (e != cudaSuccess) return e;
     k_box_partial<<<nb, kRedBlock, 0, s>>>(x, nrm, n, parts, zero_normals_ok);
     k_box_final<<<1, kRedBlock, 0, s>>>(parts, nb, parts + nb);
@@ -1129,16 +1129,46 @@ cudaError_t reduce_box(const float *x, const float *nrm, int64_t n, cudaStream_t
     return cudaGetLastError();
 }
 
+// Kernels one sort of n keys launches, for the launch counter: read off a capture
+// of the same call, which is not run, when n changes.
+int64_t sort_launches(void *tmp, size_t tb, unsigned *code, unsigned *code2, int *idx, int *idx2, int n,
+                      cudaStream_t s) {
+    thread_local int last_n = -1;
+    thread_local int64_t last = 0;
+    if (n == last_n) return last;
+    cudaGraph_t g = nullptr;
+    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return 0;
+    const cudaError_t es = cub::DeviceRadixSort::SortPairs(tmp, tb, code, code2, idx, idx2, n, 0, 30, s);
+    if (cudaStreamEndCapture(s, &g) != cudaSuccess || es != cudaSuccess) {
+        cudaGetLastError();
+        if (g) cudaGraphDestroy(g);
+        return 0;
+    }
+    size_t nn = 0;
+    cudaGraphGetNodes(g, nullptr, &nn);
+    std::vector<cudaGraphNode_t> nodes(nn);
+    if (nn) cudaGraphGetNodes(g, nodes.data(), &nn);
+    int64_t k = 0;
+    for (size_t i = 0; i < nn; ++i) {
+        cudaGraphNodeType ty;
+        if (cudaGraphNodeGetType(nodes[i], &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel) ++k;
+    }
+    cudaGraphDestroy(g);
+    last_n = n;
+    last = k;
+    return k;
+}
+
 // Morton order of n points: returns the permutation (device, caller frees).
 cudaError_t morton_order(const float *x, int64_t n, const BoxResult &bx, cudaStream_t s, int **order_out) {
     unsigned *code = nullptr, *code2 = nullptr;
     int *idx = nullptr, *idx2 = nullptr;
     void *tmp = nullptr;
     size_t tb = 0;
-    cudaError_t e = cudaMallocAsync(&code, 4 * n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&code2, 4 * n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&idx, 4 * n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&idx2, 4 * n, s);
+    cudaError_t e = pool_alloc(&code, 4 * n, s);
+    if (e == cudaSuccess) e = pool_alloc(&code2, 4 * n, s);
+    if (e == cudaSuccess) e = pool_alloc(&idx, 4 * n, s);
+    if (e == cudaSuccess) e = pool_alloc(&idx2, 4 * n, s);
     if (e == cudaSuccess) {
         float3 lo = make_float3(bx.lo[0], bx.lo[1], bx.lo[2]);
         float ext[3];
@@ -1149,32 +1179,10 @@ cudaError_t morton_order(const float *x, int64_t n, const BoxResult &bx, cudaStr
         counters().launches += 1;
         e = cub::DeviceRadixSort::SortPairs(nullptr, tb, code, code2, idx, idx2, (int)n, 0, 30, s);
     }
-    if (e == cudaSuccess) e = cudaMallocAsync(&tmp, tb > 0 ? tb : 16, s);
+    if (e == cudaSuccess) e = pool_alloc(&tmp, tb > 0 ? tb : 16, s);
     if (e == cudaSuccess) {
-        // The sort is captured into a graph so its kernel launches can be counted exactly.
-        cudaGraph_t g = nullptr;
-        cudaGraphExec_t ge = nullptr;
-        e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            const cudaError_t es = cub::DeviceRadixSort::SortPairs(tmp, tb, code, code2, idx, idx2, (int)n, 0, 30, s);
-            e = cudaStreamEndCapture(s, &g);
-            if (es != cudaSuccess) e = es;
-        }
-        if (e == cudaSuccess) {
-            size_t nn = 0;
-            cudaGraphGetNodes(g, nullptr, &nn);
-            std::vector<cudaGraphNode_t> nodes(nn);
-            if (nn) cudaGraphGetNodes(g, nodes.data(), &nn);
-            for (size_t k = 0; k < nn; ++k) {
-                cudaGraphNodeType ty;
-                if (cudaGraphNodeGetType(nodes[k], &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel)
-                    counters().launches += 1;
-            }
-            e = cudaGraphInstantiate(&ge, g, 0);
-        }
-        if (e == cudaSuccess) e = cudaGraphLaunch(ge, s);
-        if (ge) cudaGraphExecDestroy(ge);
-        if (g) cudaGraphDestroy(g);
+        counters().launches += sort_launches(tmp, tb, code, code2, idx, idx2, (int)n, s);
+        e = cub::DeviceRadixSort::SortPairs(tmp, tb, code, code2, idx, idx2, (int)n, 0, 30, s);
     }
     if (tmp) cudaFreeAsync(tmp, s);
     if (code) cudaFreeAsync(code, s);
@@ -1213,9 +1221,9 @@ cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cuda
     int *order = nullptr;
     e = morton_order(q_dev, n, bx, s, &order);
     if (e != cudaSuccess) return e;
-    e = cudaMalloc(&t->pts, sizeof(float4) * n);
-    if (e == cudaSuccess && n_dev) e = cudaMalloc(&t->nrm, sizeof(float4) * n);
-    if (e == cudaSuccess) e = cudaMalloc(&t->nodes, sizeof(float4) * 4 * ((size_t)L + ((wide_leaf(L) + L + 7) / 8) * 8));
+    e = pool_alloc(&t->pts, sizeof(float4) * n, s);
+    if (e == cudaSuccess && n_dev) e = pool_alloc(&t->nrm, sizeof(float4) * n, s);
+    if (e == cudaSuccess) e = pool_alloc(&t->nodes, sizeof(float4) * 4 * ((size_t)L + ((wide_leaf(L) + L + 7) / 8) * 8), s);
     if (e == cudaSuccess) {
         t->obb = t->nodes + 4 * (size_t)L;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q_dev, n_dev, order, n, t->pts, t->nrm);
@@ -1270,14 +1278,14 @@ __global__ void k_encode16(const float4 *__restrict__ pts, const float4 *__restr
 cudaError_t build_fp16_storage(TargetDev *t, cudaStream_t s) {
     if (t->pts16) return cudaSuccess;
     ushort4 *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, sizeof(ushort4) * (size_t)t->n);
+    cudaError_t e = pool_alloc(&p, sizeof(ushort4) * (size_t)t->n, s);
     if (e != cudaSuccess) return e;
     k_encode16<<<(unsigned)((t->n + 255) / 256), 256, 0, s>>>(t->pts, t->nodes, (int)t->n, t->L, p);
     counters().launches += 1;
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
-        cudaFree(p);
+        cudaFreeAsync(p, s);
         return e;
     }
     t->pts16 = p;
@@ -1309,10 +1317,10 @@ cudaError_t target_nu_stats(TargetDev *t, cudaStream_t s) {
     }
     double *sd = nullptr, *sh = nullptr, *out = nullptr;
     MedianState *mst = nullptr;
-    cudaError_t e = cudaMallocAsync(&sd, sizeof(double) * t->n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&mst, sizeof(MedianState), s);
-    if (e == cudaSuccess && t->has_normals) e = cudaMallocAsync(&sh, sizeof(double) * t->n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&out, 3 * sizeof(double), s);
+    cudaError_t e = pool_alloc(&sd, sizeof(double) * t->n, s);
+    if (e == cudaSuccess) e = pool_alloc(&mst, sizeof(MedianState), s);
+    if (e == cudaSuccess && t->has_normals) e = pool_alloc(&sh, sizeof(double) * t->n, s);
+    if (e == cudaSuccess) e = pool_alloc(&out, 3 * sizeof(double), s);
     int *flag = reinterpret_cast<int *>(out + 2);
     if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, 3 * sizeof(double), s);
     if (e == cudaSuccess) {
@@ -1358,8 +1366,8 @@ cudaError_t estimate_normals(const TargetDev *t, int k, const double viewpoint[3
     const int K = (int)std::min<int64_t>(k, t->n);
     double *cov = nullptr;
     int *flag = nullptr;
-    cudaError_t e = cudaMallocAsync(&cov, sizeof(double) * 6 * (size_t)t->n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&flag, sizeof(int), s);
+    cudaError_t e = pool_alloc(&cov, sizeof(double) * 6 * (size_t)t->n, s);
+    if (e == cudaSuccess) e = pool_alloc(&flag, sizeof(int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), s);
     if (e == cudaSuccess) {
         const Index ix = make_index(*t);

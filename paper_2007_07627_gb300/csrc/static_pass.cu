@@ -22,13 +22,12 @@ using fricp::PairState;
 constexpr int64_t kStaticMaxPoints = 32768;                        // largest m accepted
 constexpr int kStaticTiles = (int)(kStaticMaxPoints / fricp::kBlock);
 constexpr size_t kStateBytes = 16384;                               // >= sizeof(PairState)
-constexpr size_t kTBytes = 256;                                     // 12 doubles, then the input flag
+constexpr size_t kFlagBytes = 256;
 constexpr size_t kPartialBytes = sizeof(double) * kStaticTiles * fricp::kMaxSums;
 constexpr size_t kPrevBytes = sizeof(int) * kStaticMaxPoints;
 constexpr size_t kSrcBytes = sizeof(float4) * kStaticMaxPoints;
-constexpr size_t kOffT = kStateBytes;
-constexpr size_t kOffFlag = kOffT + 128;                            // int: a source coordinate is NaN/Inf
-constexpr size_t kOffPartial = kOffT + kTBytes;
+constexpr size_t kOffFlag = kStateBytes;                            // int: a source coordinate is NaN/Inf
+constexpr size_t kOffPartial = kOffFlag + kFlagBytes;
 constexpr size_t kOffPrev = kOffPartial + kPartialBytes;
 constexpr size_t kOffSrc = kOffPrev + kPrevBytes;
 constexpr size_t kScratchBytes = kOffSrc + kSrcBytes;               // about 0.7 MB
@@ -103,7 +102,6 @@ extern "C" fricp_status fricp_eval_pass_static(const fricp_target *target, const
     if (st != FRICP_OK) return st;
     const cudaStream_t s = (cudaStream_t)stream;
     PairState *st_dev = reinterpret_cast<PairState *>(base);
-    double *T_dev = reinterpret_cast<double *>(base + kOffT);
     double *partial = reinterpret_cast<double *>(base + kOffPartial);
     int *prev = reinterpret_cast<int *>(base + kOffPrev);
     int *bad_dev = reinterpret_cast<int *>(base + kOffFlag);
@@ -116,17 +114,12 @@ extern "C" fricp_status fricp_eval_pass_static(const fricp_target *target, const
     const double c[3] = {center ? center[0] : 0.0, center ? center[1] : 0.0, center ? center[2] : 0.0};
     PairState h = fricp::host::initial_state(prm, m, ntiles, scale, c, 1.0, 0);
     h.nu = fricp::variant_robust(variant) ? nu : 1.0;
-    double T12[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int k = 0; k < 3; ++k) T12[3 * r + k] = T_normalized[4 * r + k];
-        T12[9 + r] = T_normalized[4 * r + 3];
-    }
+    fricp::host::setup_eval(&h, T_normalized);
     // Every region the pass reads is rewritten here, so nothing from the last
-    // call leaks in: the whole state (its last-block counter included), T, the
+    // call leaks in: the whole state (its last-block counter included), the
     // input flag, the correspondences (-1: none) and the packed source. Tile
     // records are written by the pass before they are read.
     cudaError_t e = cudaMemcpyAsync(st_dev, &h, sizeof(h), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(T_dev, T12, sizeof(T12), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(bad_dev, 0, sizeof(int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(prev, 0xff, sizeof(int) * m, s);
     if (e == cudaSuccess) {
@@ -134,7 +127,6 @@ extern "C" fricp_status fricp_eval_pass_static(const fricp_target *target, const
         fricp::counters().launches += 1;
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = fricp::launch_setup_eval_xi(st_dev, T_dev, s);
     fricp::StepArgs a;
     a.st = st_dev;
     a.ix = fricp::make_index(td);
@@ -150,7 +142,7 @@ extern "C" fricp_status fricp_eval_pass_static(const fricp_target *target, const
     if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return static_fail(FRICP_ECUDA, cudaGetErrorString(e));
-    fricp::counters().h2d += sizeof(h) + sizeof(T12);
+    fricp::counters().h2d += sizeof(h);
     fricp::counters().d2h += sizeof(r) + sizeof(int);
     if (bad) return static_fail(FRICP_EINVAL, "p_xyz has NaN or Inf");
     for (int i = 0; i < 48; ++i) out[i] = r.eval_out[i];

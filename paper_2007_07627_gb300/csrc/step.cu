@@ -226,30 +226,8 @@ __global__ void __launch_bounds__(kCloseBlock) k_closest(Index ix, ClosestArgs a
     }
 }
 
-// Single-evaluation set-up for fricp_eval_pass: T is normalised (R, t). One warp.
 __global__ void __launch_bounds__(32) k_after_init(PairState *st, const double *median) {
     if (threadIdx.x == 0) start_after_init(st, *median);   // nu_max and the first stage, as after a block median
-}
-
-__global__ void __launch_bounds__(32) k_setup_eval(PairState *gst, const double *T) {
-    __shared__ double sh[kTeamScratch];
-    if (threadIdx.x >= kTeamLanes) return;
-    const Team tm{sh};
-    PairState own;
-    load_state(tm, gst, &own);
-    PairState *st = &own;
-    double Tn[12];
-    for (int i = 0; i < 12; ++i) Tn[i] = T[i];
-    if (fricp::variant_p2pl(st->variant)) {
-        double xi[6];
-        log_state_T(tm, Tn, xi);
-        request_eval_xi(tm, st, xi, 1);
-    } else {
-        request_eval_state_T(tm, st, Tn, 1);
-    }
-    st->phase = PH_EVAL;
-    set_head_cache(tm, st);
-    store_state(tm, st, gst);
 }
 
 }  // namespace
@@ -311,7 +289,7 @@ cudaError_t launch_closest(const TargetDev *t, const float *p_dev, int64_t m, co
     // scratch: cell counts, then per query its cell and rank, then the dealt queries
     char *scr = nullptr;
     const size_t cell_b = sizeof(int) * kCells, rank_b = (sizeof(int2) * (size_t)m + 15) / 16 * 16;
-    if (m >= kSortMin && cudaMallocAsync(&scr, cell_b + rank_b + sizeof(float4) * (size_t)m, s) != cudaSuccess) {
+    if (m >= kSortMin && pool_alloc(&scr, cell_b + rank_b + sizeof(float4) * (size_t)m, s) != cudaSuccess) {
         cudaGetLastError();   // no room: search them as they come
         scr = nullptr;
     }
@@ -346,12 +324,6 @@ cudaError_t launch_closest(const TargetDev *t, const float *p_dev, int64_t m, co
 
 cudaError_t launch_after_init(PairState *st, const double *median_dev, cudaStream_t s) {
     k_after_init<<<1, 32, 0, s>>>(st, median_dev);
-    counters().launches += 1;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_setup_eval_xi(PairState *st, const double *T_normalized12, cudaStream_t s) {
-    k_setup_eval<<<1, 32, 0, s>>>(st, T_normalized12);
     counters().launches += 1;
     return cudaGetLastError();
 }
