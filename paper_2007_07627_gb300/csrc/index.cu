@@ -750,15 +750,20 @@ __global__ void __launch_bounds__(kKnnBlock) k_knn6_tile(Index ix, double *__res
 // original index); the normal is the eigenvector of the smallest eigenvalue of
 // the neighbourhood's covariance about its centroid, turned towards a viewpoint.
 //
-// k_knn_cov: one warp per point, the traversal of warp_knn6. The warp keeps the
-// sorted k nearest one entry per lane (lane s holds the s-th nearest), inserts a
-// candidate with one ballot and one shift, and prunes in float against the k-th
-// distance rounded up. Candidate distances are FP64 without fused
-// multiply-adds, so the order is that of a plain evaluation of
-// (dx^2 + dy^2) + dz^2. Writes the 6 covariance entries per point.
+// k_normals: a warp takes up to 32 Morton-consecutive points.
+//   1. For each of them the whole warp finds the K nearest by float distance
+//      (near_knn: the traversal of warp_knn6, the sorted list one entry per
+//      lane, new buckets merged 32 candidates at a time). Float distances have a
+//      relative error below 4e-7, so the set is the exact one unless the
+//      (K+1)-th lies within 2e-6 of the K-th; those points (ties, and about one
+//      in 10^4 otherwise) are searched again with FP64 distances (warp_knn_k).
+//   2. Each lane takes one point: the covariance of its neighbours in FP64 and
+//      its smallest eigenvector (smallest_axis).
+// GB300 issues an FP64 warp instruction once in 64 cycles however many lanes it
+// has, so FP64 work spread over a warp per point (distances, list comparisons,
+// covariance sums, 3.0 ms of k_knn_cov for 100,000 points) was the bound; with a
+// point per lane it is 1/32 of that, and the search is bound by issue slots.
 // ---------------------------------------------------------------------------
-constexpr int kMaxNormalK = 32;
-
 __device__ __forceinline__ double exact_d2(float4 q, const float xq[3]) {
     const double a0 = (double)q.x - (double)xq[0], a1 = (double)q.y - (double)xq[1], a2 = (double)q.z - (double)xq[2];
     return __dadd_rn(__dadd_rn(__dmul_rn(a0, a0), __dmul_rn(a1, a1)), __dmul_rn(a2, a2));
@@ -795,7 +800,9 @@ __device__ __forceinline__ void topk_scan(const Index &ix, const float xq[3], To
         cm &= cm - 1u;
         const double dv = __shfl_sync(FULL, d, src);
         const int ov = __shfl_sync(FULL, o, src), jv = __shfl_sync(FULL, j, src);
-        const bool greater = lane < K && (t.d > dv || (t.d == dv && t.o > ov));
+        // non-negative doubles order as their bits: no FP64 comparison
+        const long long td = __double_as_longlong(t.d), cd = __double_as_longlong(dv);
+        const bool greater = lane < K && (td > cd || (td == cd && t.o > ov));
         const unsigned gm = __ballot_sync(FULL, greater);
         if (gm == 0u) continue;   // not among the K nearest
         const int pos = __ffs(gm) - 1;
@@ -814,8 +821,9 @@ __device__ __forceinline__ void topk_scan(const Index &ix, const float xq[3], To
     }
 }
 
-// Returns false if the stack would overflow.
-__device__ bool warp_knn_k(const Index &ix, int i, const float xq[3], int K, TopK &t, int *stk) {
+// The K nearest by (FP64 distance, original index). Returns false if the stack
+// would overflow.
+__device__ __noinline__ bool warp_knn_k(const Index &ix, int i, const float xq[3], int K, TopK &t, int *stk) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
@@ -902,66 +910,157 @@ __device__ bool warp_knn_k(const Index &ix, int i, const float xq[3], int K, Top
     return true;
 }
 
-__global__ void __launch_bounds__(kKnnBlock) k_knn_cov(Index ix, int K, double *__restrict__ cov,
-                                                       int *__restrict__ overflow) {
-    __shared__ int s_stk[kKnnBlock / 32][kWarpStack];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int wpb = kKnnBlock / 32;
-    for (int i = blockIdx.x * wpb + w; i < ix.n; i += gridDim.x * wpb) {
-        const float4 qi = __ldg(ix.pts + i);
-        const float xq[3] = {qi.x, qi.y, qi.z};
-        TopK t;
-        if (!warp_knn_k(ix, i, xq, K, t, s_stk[w])) {
-            if (lane == 0) *overflow = 1;
-            continue;
-        }
-        // centroid and covariance of the K neighbours (lanes 0..K-1), FP64 warp sums
-        double p[3] = {0.0, 0.0, 0.0};
-        if (lane < K) {
-            const float4 q = __ldg(ix.pts + t.j);
-            p[0] = q.x;
-            p[1] = q.y;
-            p[2] = q.z;
-        }
-        double c[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            double v = p[a];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            c[a] = v / (double)K;
-        }
-        double e[6] = {0, 0, 0, 0, 0, 0};
-        if (lane < K) {
-            const double x = p[0] - c[0], y = p[1] - c[1], z = p[2] - c[2];
-            e[0] = x * x;
-            e[1] = x * y;
-            e[2] = x * z;
-            e[3] = y * y;
-            e[4] = y * z;
-            e[5] = z * z;
-        }
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e[a] += __shfl_xor_sync(0xffffffffu, e[a], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int a = 0; a < 6; ++a) cov[6 * (size_t)i + a] = e[a] / (double)K;
-        }
+// The 32 nearest points of a query by float distance, lane s the s-th.
+struct NearK {
+    float d;
+    int j;
+    float bound;   // the K-th distance
+    float spill;   // smallest distance that left the list
+};
+
+// Compare-exchange with lane ^ s, the smaller distance to the lower lane when
+// `up`. Equal distances stay where they are, in both lanes.
+__device__ __forceinline__ void near_exchange(float &d, int &j, int s, bool up) {
+    const unsigned FULL = 0xffffffffu;
+    const float od = __shfl_xor_sync(FULL, d, s);
+    const int oj = __shfl_xor_sync(FULL, j, s);
+    const bool keep_min = ((threadIdx.x & s) == 0) == up;
+    if (keep_min ? od < d : od > d) {
+        d = od;
+        j = oj;
     }
 }
 
-// Eigenvector of the smallest eigenvalue of each 3x3 covariance (cyclic Jacobi
-// in FP64), turned so that n . (viewpoint - q) >= 0, written at the point's
-// original index.
-__global__ void k_normal_from_cov(Index ix, const double *__restrict__ cov, double v0, double v1, double v2,
-                                  float *__restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ix.n) return;
+__device__ __forceinline__ void near_scan(const Index &ix, const float xq[3], NearK &t, int K, int na, int nb,
+                                          bool two) {
+    const unsigned FULL = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31;
+    float d = INF;
+    int j = -1;
+    if (lane < 16 || two) {
+        j = ((lane < 16 ? na : nb) - ix.L) * kLeaf + (lane & 15);
+        if (j < ix.n) {
+            const float4 q = __ldg(ix.pts + j);
+            const float fx = q.x - xq[0], fy = q.y - xq[1], fz = q.z - xq[2];
+            d = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
+            if (!(d * kShrink <= t.bound)) d = INF;
+        }
+    }
+    unsigned cm = __ballot_sync(FULL, d < INF);
+    if (cm == 0u) return;
+    if (__popc(cm) <= 3) {   // a few: insert one by one
+        while (cm) {
+            const int src = __ffs(cm) - 1;
+            cm &= cm - 1u;
+            const float dv = __shfl_sync(FULL, d, src);
+            const int jv = __shfl_sync(FULL, j, src);
+            const unsigned gm = __ballot_sync(FULL, t.d > dv);
+            const float ud = __shfl_up_sync(FULL, t.d, 1);
+            const int uj = __shfl_up_sync(FULL, t.j, 1);
+            t.spill = fminf(t.spill, gm == 0u ? dv : __shfl_sync(FULL, t.d, 31));
+            if (gm == 0u) continue;
+            const int pos = __ffs(gm) - 1;
+            if (lane >= pos) {
+                t.d = lane == pos ? dv : ud;
+                t.j = lane == pos ? jv : uj;
+            }
+        }
+    } else {   // sort the 32 descending, merge with the ascending list, keep the lower half
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+            for (int o = k >> 1; o > 0; o >>= 1) near_exchange(d, j, o, (lane & k) != 0);
+        float out = t.d > d ? t.d : d;
+        if (d < t.d) {
+            t.d = d;
+            t.j = j;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) near_exchange(t.d, t.j, o, true);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) out = fminf(out, __shfl_xor_sync(FULL, out, o));
+        t.spill = fminf(t.spill, out);
+    }
+    t.bound = __shfl_sync(FULL, t.d, K - 1);
+}
+
+// The K nearest of point i in lanes 0 .. K-1. Returns 0 if they are the exact K,
+// 1 if float distances cannot tell, 2 if the stack would overflow.
+__device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3], int K, NearK &t, int *stk) {
+    const unsigned FULL = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float zero[3] = {0.0f, 0.0f, 0.0f};
+    t.d = t.bound = t.spill = INF;
+    t.j = -1;
+    const int depth = 31 - __clz(ix.L);
+    const int start = ix.L + i / kLeaf;
+    near_scan(ix, xq, t, K, start, start ^ 1, depth > 0);   // the point's bucket and its sibling first
+    int sp;
+    {
+        int c = 0;
+        bool pass = false;
+        if (lane < depth - 1) {
+            c = (start >> (depth - 1 - lane)) ^ 1;
+            pass = box_d2(__ldg(ix.nodes + 2 * c), __ldg(ix.nodes + 2 * c + 1), xq, zero) * kShrink <= t.bound;
+        }
+        const unsigned m = __ballot_sync(FULL, pass);
+        if (pass) stk[__popc(m & below)] = c;
+        sp = __popc(m);
+    }
+    __syncwarp();
+    while (sp > 0) {
+        const int k = min(32, sp);
+        const int node = (lane < k) ? stk[sp - 1 - lane] : 0;
+        sp -= k;
+        __syncwarp();
+        // inner nodes at least two levels above the buckets expand to four grandchildren, others to two children
+        int c0 = 0, nc = 0;
+        bool leaf_ok = false;
+        if (node != 0) {
+            if (node < ix.L) {
+                const bool deep = 2 * node < ix.L;
+                c0 = deep ? 4 * node : 2 * node;
+                nc = deep ? 4 : 2;
+            } else {
+                leaf_ok = box_d2(__ldg(ix.nodes + 2 * node), __ldg(ix.nodes + 2 * node + 1), xq, zero) * kShrink
+                              <= t.bound &&
+                          obb_d2(obb_at(ix.obb, node - ix.L + ix.leaf0), xq, zero) * kObbShrink <= t.bound;
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            bool ok = false;
+            if (g < nc)
+                ok = box_d2(__ldg(ix.nodes + 2 * (c0 + g)), __ldg(ix.nodes + 2 * (c0 + g) + 1), xq, zero) * kShrink <=
+                     t.bound;
+            const unsigned mg = __ballot_sync(FULL, ok);
+            if (sp + __popc(mg) > kWarpStack) return 2;
+            if (ok) stk[sp + __popc(mg & below)] = c0 + g;
+            sp += __popc(mg);
+        }
+        unsigned lm = __ballot_sync(FULL, leaf_ok);
+        while (lm) {   // two buckets per pass: lanes 0-15 and 16-31
+            const int la = __ffs(lm) - 1;
+            lm &= lm - 1u;
+            const bool two = lm != 0u;
+            const int lb = two ? __ffs(lm) - 1 : la;
+            if (two) lm &= lm - 1u;
+            const int na = __shfl_sync(FULL, node, la), nb = __shfl_sync(FULL, node, lb);
+            near_scan(ix, xq, t, K, na, nb, two);
+        }
+        __syncwarp();
+    }
+    const float next = K < 32 ? __shfl_sync(FULL, t.d, K & 31) : t.spill;
+    return !(t.bound < INF) || (next <= t.bound * kTieWindow && next < INF) ? 1 : 0;   // not finite: distances beyond float
+}
+
+// Eigenvector of the smallest eigenvalue of the symmetric matrix e (xx, xy, xz,
+// yy, yz, zz) by cyclic Jacobi rotations in FP64.
+__device__ __noinline__ void jacobi_axis(const double e[6], double n[3]) {
     double a[3][3], V[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
-    const double *e = cov + 6 * (size_t)i;
     a[0][0] = e[0];
     a[0][1] = a[1][0] = e[1];
     a[0][2] = a[2][0] = e[2];
@@ -999,12 +1098,112 @@ __global__ void k_normal_from_cov(Index ix, const double *__restrict__ cov, doub
     int m = 0;
     if (a[1][1] < a[m][m]) m = 1;
     if (a[2][2] < a[m][m]) m = 2;
-    double n[3] = {V[0][m], V[1][m], V[2][m]};
+    for (int k = 0; k < 3; ++k) n[k] = V[k][m];
+}
+
+// The same vector (any length) when the two smaller eigenvalues are apart: float
+// Jacobi rotations, then two Rayleigh quotient steps in FP64, n <- adj(A - s I) n
+// with s = n.A n / n.n. A step cubes the float error (below 1e-2 where the gap
+// exceeds 1e-4 of the largest eigenvalue), so two give the FP64 eigenvector, in
+// about 100 FP64 instructions instead of 1,300. Smaller gaps take jacobi_axis.
+__device__ __forceinline__ void smallest_axis(const double e[6], double n[3]) {
+    const double sc = e[0] + e[3] + e[5];
+    const float is = 1.0f / (float)sc;
+    const float f[6] = {(float)e[0] * is, (float)e[1] * is, (float)e[2] * is,
+                        (float)e[3] * is, (float)e[4] * is, (float)e[5] * is};
+    float A[3][3] = {{f[0], f[1], f[2]}, {f[1], f[3], f[4]}, {f[2], f[4], f[5]}}, V[3][3];
+    jacobi3f(A, V);
+    const float l0 = A[0][0], l1 = A[1][1], l2 = A[2][2];
+    const float lo = fminf(l0, fminf(l1, l2)), hi = fmaxf(l0, fmaxf(l1, l2));
+    const float mid = fmaxf(fminf(l0, l1), fminf(fmaxf(l0, l1), l2));
+    if (!(mid - lo > 1e-4f * hi) || !(is > 1e-30f && is < 1e30f)) {
+        jacobi_axis(e, n);
+        return;
+    }
+    const bool m1 = l1 == lo, m2 = l2 == lo;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) n[k] = (double)(m2 ? V[k][2] : (m1 ? V[k][1] : V[k][0]));
+    const double ds = (double)is;
+    const double xx = e[0] * ds, xy = e[1] * ds, xz = e[2] * ds, yy = e[3] * ds, yz = e[4] * ds, zz = e[5] * ds;
+#pragma unroll
+    for (int step = 0; step < 2; ++step) {
+        const double n2 = fma(n[2], n[2], fma(n[1], n[1], n[0] * n[0]));
+        double u[3] = {fma(xz, n[2], fma(xy, n[1], xx * n[0])), fma(yz, n[2], fma(yy, n[1], xy * n[0])),
+                       fma(zz, n[2], fma(yz, n[1], xz * n[0]))};
+        const double inv = (double)(1.0f / (float)n2);   // the quotient to float accuracy of |n|^2, refined once
+        const double r = inv * fma(-n2, inv, 2.0);
+        const double s = fma(n[2], u[2], fma(n[1], u[1], n[0] * u[0])) * r;
+        const double a = xx - s, b = yy - s, c = zz - s;
+        const double c00 = fma(b, c, -(yz * yz)), c01 = fma(xz, yz, -(xy * c)), c02 = fma(xy, yz, -(xz * b));
+        const double c11 = fma(a, c, -(xz * xz)), c12 = fma(xy, xz, -(a * yz)), c22 = fma(a, b, -(xy * xy));
+        u[0] = fma(c02, n[2], fma(c01, n[1], c00 * n[0]));
+        u[1] = fma(c12, n[2], fma(c11, n[1], c01 * n[0]));
+        u[2] = fma(c22, n[2], fma(c12, n[1], c02 * n[0]));
+        // back to about unit length (any positive factor does)
+        const float q = (float)fma(u[2], u[2], fma(u[1], u[1], u[0] * u[0]));
+        const double g = (double)rsqrtf(q);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) n[k] = u[k] * g;
+    }
+}
+
+// Normals of `per_warp` (a power of two up to 32) Morton-consecutive points per
+// warp, turned so that n . (viewpoint - q) >= 0, written at the original index.
+__global__ void __launch_bounds__(kKnnBlock) k_normals(Index ix, int K, int per_warp, double v0, double v1, double v2,
+                                                       float *__restrict__ out, int *__restrict__ overflow) {
+    __shared__ int s_stk[kKnnBlock / 32][kWarpStack];
+    __shared__ int s_nbr[kKnnBlock / 32][32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i0 = ((int64_t)blockIdx.x * (kKnnBlock / 32) + w) * per_warp;
+    for (int p = 0; p < per_warp; ++p) {
+        const int64_t i = i0 + p;
+        if (i >= ix.n) break;   // uniform in the warp
+        const float4 qi = __ldg(ix.pts + i);
+        const float xq[3] = {qi.x, qi.y, qi.z};
+        NearK t;
+        int rc = near_knn(ix, (int)i, xq, K, t, s_stk[w]);
+        __syncwarp();
+        if (rc == 1) {
+            TopK e;
+            rc = warp_knn_k(ix, (int)i, xq, K, e, s_stk[w]) ? 0 : 2;
+            t.j = e.j;
+        }
+        if (rc == 2 && lane == 0) *overflow = 1;
+        s_nbr[w][p][lane] = rc == 2 ? (int)i : t.j;
+        __syncwarp();
+    }
+    const int64_t i = i0 + lane;
+    if (lane >= per_warp || i >= ix.n) return;
+    const float4 qi = __ldg(ix.pts + i);
+    const double x = qi.x, y = qi.y, z = qi.z;
+    // sums of the differences to the point and of their products
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, e[6] = {0, 0, 0, 0, 0, 0};
+    for (int k = 0; k < K; ++k) {
+        const float4 q = __ldg(ix.pts + s_nbr[w][lane][k]);
+        const double d0 = (double)q.x - x, d1 = (double)q.y - y, d2 = (double)q.z - z;
+        s0 += d0;
+        s1 += d1;
+        s2 += d2;
+        e[0] = fma(d0, d0, e[0]);
+        e[1] = fma(d0, d1, e[1]);
+        e[2] = fma(d0, d2, e[2]);
+        e[3] = fma(d1, d1, e[3]);
+        e[4] = fma(d1, d2, e[4]);
+        e[5] = fma(d2, d2, e[5]);
+    }
+    const double ik = 1.0 / (double)K;
+    e[0] = fma(-s0 * ik, s0, e[0]);
+    e[1] = fma(-s0 * ik, s1, e[1]);
+    e[2] = fma(-s0 * ik, s2, e[2]);
+    e[3] = fma(-s1 * ik, s1, e[3]);
+    e[4] = fma(-s1 * ik, s2, e[4]);
+    e[5] = fma(-s2 * ik, s2, e[5]);
+    double n[3];
+    smallest_axis(e, n);
     const double inv = 1.0 / sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-    const float4 q = __ldg(ix.pts + i);
-    const double side = n[0] * (v0 - (double)q.x) + n[1] * (v1 - (double)q.y) + n[2] * (v2 - (double)q.z);
+    const double side = n[0] * (v0 - x) + n[1] * (v1 - y) + n[2] * (v2 - z);
     const double sg = side < 0.0 ? -inv : inv;
-    const int o = __float_as_int(q.w);
+    const int o = __float_as_int(qi.w);
     out[3 * (size_t)o] = (float)(n[0] * sg);
     out[3 * (size_t)o + 1] = (float)(n[1] * sg);
     out[3 * (size_t)o + 2] = (float)(n[2] * sg);
@@ -1364,29 +1563,27 @@ cudaError_t target_nu_stats(TargetDev *t, cudaStream_t s) {
 cudaError_t estimate_normals(const TargetDev *t, int k, const double viewpoint[3], float *out_dev, cudaStream_t s,
                              int *overflow_out) {
     const int K = (int)std::min<int64_t>(k, t->n);
-    double *cov = nullptr;
     int *flag = nullptr;
-    cudaError_t e = pool_alloc(&cov, sizeof(double) * 6 * (size_t)t->n, s);
-    if (e == cudaSuccess) e = pool_alloc(&flag, sizeof(int), s);
+    cudaError_t e = pool_alloc(&flag, sizeof(int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), s);
     if (e == cudaSuccess) {
         const Index ix = make_index(*t);
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int64_t blocks = std::min<int64_t>((t->n + kKnnBlock / 32 - 1) / (kKnnBlock / 32),
-                                                 (int64_t)(sms > 0 ? sms : 152) * 16);
-        k_knn_cov<<<(unsigned)blocks, kKnnBlock, 0, s>>>(ix, K, cov, flag);
-        k_normal_from_cov<<<(unsigned)((t->n + 255) / 256), 256, 0, s>>>(ix, cov, viewpoint[0], viewpoint[1],
-                                                                         viewpoint[2], out_dev);
-        counters().launches += 2;
+        // 32 points per warp use the FP64 units best; fewer while that leaves an SM less than 16 warps
+        int per_warp = 32;
+        while (per_warp > 4 && t->n / per_warp < (int64_t)16 * (sms > 0 ? sms : 152)) per_warp /= 2;
+        const int64_t per_block = (int64_t)per_warp * (kKnnBlock / 32);
+        k_normals<<<(unsigned)((t->n + per_block - 1) / per_block), kKnnBlock, 0, s>>>(
+            ix, K, per_warp, viewpoint[0], viewpoint[1], viewpoint[2], out_dev, flag);
+        counters().launches += 1;
         e = cudaGetLastError();
     }
     int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, s);
     counters().d2h += sizeof(int);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (cov) cudaFreeAsync(cov, s);
     if (flag) cudaFreeAsync(flag, s);
     *overflow_out = h;
     return e;
