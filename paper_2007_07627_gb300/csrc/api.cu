@@ -92,7 +92,7 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
             if (timing) cudaEventRecord(iev[0], s);
             e = fricp::launch_step(a, variant, prec, ntiles, s, timing ? iev[1] : nullptr);
             if (timing) cudaEventRecord(iev[2], s);
-            if (e == cudaSuccess) e = fricp::launch_median(a.resid, (int)init_m, mscr.p, med, s);
+            if (e == cudaSuccess) e = fricp::launch_median(a.resid, nullptr, (int)init_m, mscr.p, med, s);
             if (e == cudaSuccess) e = fricp::launch_after_init(a.st, med, s);
             if (e != cudaSuccess) rs = cuda_fail(e, "launching the initial pass");
             steps = 1;

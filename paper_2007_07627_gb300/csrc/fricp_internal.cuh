@@ -637,10 +637,11 @@ cudaError_t launch_closest(const TargetDev *t, const float *p_dev, int64_t m, co
 cudaError_t launch_step(const StepArgs &a, int variant, int prec, int ntiles, cudaStream_t s,
                         cudaEvent_t mid = nullptr);
 // Median of n non-negative doubles (the mean of the two middle order
-// statistics, exact) by a grid-wide 8-bit radix select; `scratch` holds
-// kMedianScratchBytes of device memory, the result lands in *out_dev.
-constexpr int kMedianScratchBytes = 4096;
-cudaError_t launch_median(const double *v, int n, void *scratch, double *out_dev, cudaStream_t s);
+// statistics, exact) by a grid-wide 8-bit radix select, of v and, when v2 is
+// given, of v2 beside it; `scratch` holds kMedianScratchBytes of device memory,
+// the results land in out_dev[0] and out_dev[1].
+constexpr int kMedianScratchBytes = 8192;
+cudaError_t launch_median(const double *v, const double *v2, int n, void *scratch, double *out_dev, cudaStream_t s);
 // After a first pass run with init_median_ext: nu_max from the median at
 // *median_dev and the first nu stage (start_after_init).
 cudaError_t launch_after_init(PairState *st, const double *median_dev, cudaStream_t s);

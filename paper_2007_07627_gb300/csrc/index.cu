@@ -561,20 +561,25 @@ __global__ void __launch_bounds__(kKnnBlock) k_knn6_stats(Index ix, double *__re
 
 // Six-neighbour statistics by tiles: a warp takes the 32 Morton-consecutive
 // target points of buckets 2g and 2g + 1, one per lane, each lane keeping its
-// own six nearest (Best6, the same (FP64 distance, index) order and float
-// pre-test as warp_knn6).
-//   1. Each lane offers the tile's other 31 points to its six: its sixth
+// own nearest.
+//   1. Each lane offers the tile's other 31 points to its list: its sixth
 //      distance is then an upper bound of its true sixth distance, and R, the
-//      largest over the lanes (rounded up to float), bounds them all.
+//      largest over the lanes, bounds them all.
 //   2. Every point within sqrt(R) of some lane's point lies within sqrt(R) of
 //      the two buckets' common box (the tree node above them), so the buckets
 //      whose box is within that distance of that box (walk from the node's path
 //      siblings, box-to-box distance, kShrink slack) hold every candidate.
-//   3. Each lane offers the points of those buckets to its six, pruning with
+//   3. Each lane offers the points of those buckets to its list, pruning with
 //      its own sixth distance.
-// The six selected are therefore the exact six of warp_knn6. A tile whose
-// bucket list does not fit (a scattered tile, or fewer than seven points in
-// it) is searched point by point with warp_knn6 instead.
+// The lists rank by float distance (tile_near7, seven entries); a tile in which
+// the seventh cannot be told from the sixth repeats it with FP64 distances
+// (tile_knn6: Best6, the order and float pre-test of warp_knn6). A tile whose
+// bucket list does not fit (scattered, or fewer than seven points in it) is left
+// to k_knn6_rest, which gives each of its points a warp.
+// With every distance and comparison in FP64, and the left-over tiles searched
+// point by point by their own warp, the FP64 pipe and a few such warps were the
+// bound (ellipsoids, 500,000 points: 2.48 ms); now 0.36 ms, issue-bound, and 0.11
+// ms for the rest.
 constexpr int kKnnCand = 192;   // candidate buckets per tile
 
 __device__ __forceinline__ float box_box_d2(float4 alo, float4 ahi, float4 blo, float4 bhi) {
@@ -593,35 +598,12 @@ __device__ __forceinline__ void knn6_offer_own(Best6 &b, float4 q, const float x
     }
 }
 
-// Returns false when the candidate list or the walk's stack would overflow.
-__device__ bool tile_knn6(const Index &ix, int g, int i, bool live, const float xq[3], Best6 &b, int *stk,
-                          int *cand) {
+// Buckets within sqrt(R) of the box of tile g (node P above buckets 2g, 2g + 1),
+// in cand; their number, or -1 when the list or the walk's stack would overflow.
+__device__ __forceinline__ int tile_candidates(const Index &ix, int g, float R, int *stk, int *cand) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    for (int s = 0; s < 6; ++s) {
-        b.d[s] = INFINITY;
-        b.o[s] = 0x7fffffff;
-        b.j[s] = -1;
-    }
-    b.bound = INFINITY;
-    const int i0 = 32 * g;
-    const float4 mine = live ? __ldg(ix.pts + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    for (int k = 1; k < 32; ++k) {   // 1. the tile's own points, nearest in Morton order first
-        const int off = (k & 1) ? (k + 1) >> 1 : -(k >> 1);   // +1, -1, +2, -2, ..., -15, +16
-        const int t = (lane + off) & 31;
-        float4 q;
-        q.x = __shfl_sync(FULL, mine.x, t);
-        q.y = __shfl_sync(FULL, mine.y, t);
-        q.z = __shfl_sync(FULL, mine.z, t);
-        q.w = __shfl_sync(FULL, mine.w, t);
-        if (live && i0 + t < ix.n) knn6_offer_own(b, q, xq, i0 + t);
-    }
-    float R = live ? b.bound : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) R = fmaxf(R, __shfl_xor_sync(FULL, R, o));
-    if (!(R < INFINITY)) return false;
-    // 2. buckets within sqrt(R) of the tile's box (node P above buckets 2g, 2g + 1)
     int depth = 0;
     while ((1 << depth) < ix.L) ++depth;
     const int P = (ix.L >> 1) + g;
@@ -670,20 +652,52 @@ __device__ bool tile_knn6(const Index &ix, int g, int i, bool live, const float 
             }
         }
         const unsigned lm = __ballot_sync(FULL, leaf);
-        if (nc + __popc(lm) > kKnnCand) return false;
+        if (nc + __popc(lm) > kKnnCand) return -1;
         if (leaf) cand[nc + __popc(lm & below)] = node;
         nc += __popc(lm);
         int base = sp;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const unsigned mq = __ballot_sync(FULL, ok[q]);
-            if (base + __popc(mq) > kWarpStack - kKnnCand) return false;
+            if (base + __popc(mq) > kWarpStack - kKnnCand) return -1;
             if (ok[q]) stk[base + __popc(mq & below)] = c[q];
             base += __popc(mq);
         }
         sp = base;
         __syncwarp();
     }
+    return nc;
+}
+
+// Returns false when the candidate list or the walk's stack would overflow.
+__device__ __noinline__ bool tile_knn6(const Index &ix, int g, int i, bool live, const float xq[3], Best6 &b, int *stk,
+                          int *cand) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    for (int s = 0; s < 6; ++s) {
+        b.d[s] = INFINITY;
+        b.o[s] = 0x7fffffff;
+        b.j[s] = -1;
+    }
+    b.bound = INFINITY;
+    const int i0 = 32 * g;
+    const float4 mine = live ? __ldg(ix.pts + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k = 1; k < 32; ++k) {   // 1. the tile's own points, nearest in Morton order first
+        const int off = (k & 1) ? (k + 1) >> 1 : -(k >> 1);   // +1, -1, +2, -2, ..., -15, +16
+        const int t = (lane + off) & 31;
+        float4 q;
+        q.x = __shfl_sync(FULL, mine.x, t);
+        q.y = __shfl_sync(FULL, mine.y, t);
+        q.z = __shfl_sync(FULL, mine.z, t);
+        q.w = __shfl_sync(FULL, mine.w, t);
+        if (live && i0 + t < ix.n) knn6_offer_own(b, q, xq, i0 + t);
+    }
+    float R = live ? b.bound : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) R = fmaxf(R, __shfl_xor_sync(FULL, R, o));
+    if (!(R < INFINITY)) return false;
+    const int nc = tile_candidates(ix, g, R, stk, cand);   // 2.
+    if (nc < 0) return false;
     // 3. every lane offers the candidates' points to its own six, bucket by
     //    bucket; a lane whose own bound the bucket's boxes exceed skips it, and
     //    the warp skips a bucket no lane needs
@@ -704,41 +718,343 @@ __device__ bool tile_knn6(const Index &ix, int g, int i, bool live, const float 
     return true;
 }
 
+// The 32 nearest points of a query by float distance, lane s the s-th.
+struct NearK {
+    float d;
+    int j;
+    float bound;   // the K-th distance
+    float spill;   // smallest distance that left the list
+};
+
+// Compare-exchange with lane ^ s, the smaller distance to the lower lane when
+// `up`. Equal distances stay where they are, in both lanes.
+__device__ __forceinline__ void near_exchange(float &d, int &j, int s, bool up) {
+    const unsigned FULL = 0xffffffffu;
+    const float od = __shfl_xor_sync(FULL, d, s);
+    const int oj = __shfl_xor_sync(FULL, j, s);
+    const bool keep_min = ((threadIdx.x & s) == 0) == up;
+    if (keep_min ? od < d : od > d) {
+        d = od;
+        j = oj;
+    }
+}
+
+__device__ __forceinline__ void near_scan(const Index &ix, const float xq[3], int skip, NearK &t, int K, int na,
+                                          int nb, bool two) {
+    const unsigned FULL = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31;
+    float d = INF;
+    int j = -1;
+    if (lane < 16 || two) {
+        j = ((lane < 16 ? na : nb) - ix.L) * kLeaf + (lane & 15);
+        if (j < ix.n && j != skip) {
+            const float4 q = __ldg(ix.pts + j);
+            const float fx = q.x - xq[0], fy = q.y - xq[1], fz = q.z - xq[2];
+            d = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
+            if (!(d * kShrink <= t.bound)) d = INF;
+        }
+    }
+    unsigned cm = __ballot_sync(FULL, d < INF);
+    if (cm == 0u) return;
+    if (__popc(cm) <= 3) {   // a few: insert one by one
+        while (cm) {
+            const int src = __ffs(cm) - 1;
+            cm &= cm - 1u;
+            const float dv = __shfl_sync(FULL, d, src);
+            const int jv = __shfl_sync(FULL, j, src);
+            const unsigned gm = __ballot_sync(FULL, t.d > dv);
+            const float ud = __shfl_up_sync(FULL, t.d, 1);
+            const int uj = __shfl_up_sync(FULL, t.j, 1);
+            t.spill = fminf(t.spill, gm == 0u ? dv : __shfl_sync(FULL, t.d, 31));
+            if (gm == 0u) continue;
+            const int pos = __ffs(gm) - 1;
+            if (lane >= pos) {
+                t.d = lane == pos ? dv : ud;
+                t.j = lane == pos ? jv : uj;
+            }
+        }
+    } else {   // sort the 32 descending, merge with the ascending list, keep the lower half
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+            for (int o = k >> 1; o > 0; o >>= 1) near_exchange(d, j, o, (lane & k) != 0);
+        float out = t.d > d ? t.d : d;
+        if (d < t.d) {
+            t.d = d;
+            t.j = j;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) near_exchange(t.d, t.j, o, true);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) out = fminf(out, __shfl_xor_sync(FULL, out, o));
+        t.spill = fminf(t.spill, out);
+    }
+    t.bound = __shfl_sync(FULL, t.d, K - 1);
+}
+
+// The K nearest of point i in lanes 0 .. K-1 (point `skip` left out). Returns 0 if they are the exact K,
+// 1 if float distances cannot tell, 2 if the stack would overflow.
+__device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3], int skip, int K, NearK &t, int *stk) {
+    const unsigned FULL = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float zero[3] = {0.0f, 0.0f, 0.0f};
+    t.d = t.bound = t.spill = INF;
+    t.j = -1;
+    const int depth = 31 - __clz(ix.L);
+    const int start = ix.L + i / kLeaf;
+    near_scan(ix, xq, skip, t, K, start, start ^ 1, depth > 0);   // the point's bucket and its sibling first
+    int sp;
+    {
+        int c = 0;
+        bool pass = false;
+        if (lane < depth - 1) {
+            c = (start >> (depth - 1 - lane)) ^ 1;
+            pass = box_d2(__ldg(ix.nodes + 2 * c), __ldg(ix.nodes + 2 * c + 1), xq, zero) * kShrink <= t.bound;
+        }
+        const unsigned m = __ballot_sync(FULL, pass);
+        if (pass) stk[__popc(m & below)] = c;
+        sp = __popc(m);
+    }
+    __syncwarp();
+    while (sp > 0) {
+        const int k = min(32, sp);
+        const int node = (lane < k) ? stk[sp - 1 - lane] : 0;
+        sp -= k;
+        __syncwarp();
+        // inner nodes at least two levels above the buckets expand to four grandchildren, others to two children
+        int c0 = 0, nc = 0;
+        bool leaf_ok = false;
+        if (node != 0) {
+            if (node < ix.L) {
+                const bool deep = 2 * node < ix.L;
+                c0 = deep ? 4 * node : 2 * node;
+                nc = deep ? 4 : 2;
+            } else {
+                leaf_ok = box_d2(__ldg(ix.nodes + 2 * node), __ldg(ix.nodes + 2 * node + 1), xq, zero) * kShrink
+                              <= t.bound &&
+                          obb_d2(obb_at(ix.obb, node - ix.L + ix.leaf0), xq, zero) * kObbShrink <= t.bound;
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            bool ok = false;
+            if (g < nc)
+                ok = box_d2(__ldg(ix.nodes + 2 * (c0 + g)), __ldg(ix.nodes + 2 * (c0 + g) + 1), xq, zero) * kShrink <=
+                     t.bound;
+            const unsigned mg = __ballot_sync(FULL, ok);
+            if (sp + __popc(mg) > kWarpStack) return 2;
+            if (ok) stk[sp + __popc(mg & below)] = c0 + g;
+            sp += __popc(mg);
+        }
+        unsigned lm = __ballot_sync(FULL, leaf_ok);
+        while (lm) {   // two buckets per pass: lanes 0-15 and 16-31
+            const int la = __ffs(lm) - 1;
+            lm &= lm - 1u;
+            const bool two = lm != 0u;
+            const int lb = two ? __ffs(lm) - 1 : la;
+            if (two) lm &= lm - 1u;
+            const int na = __shfl_sync(FULL, node, la), nb = __shfl_sync(FULL, node, lb);
+            near_scan(ix, xq, skip, t, K, na, nb, two);
+        }
+        __syncwarp();
+    }
+    const float next = K < 32 ? __shfl_sync(FULL, t.d, K & 31) : t.spill;
+    return !(t.bound < INF) || (next <= t.bound * kTieWindow && next < INF) ? 1 : 0;   // not finite: distances beyond float
+}
+
+// The same selection by float distance: each lane keeps its seven nearest, sorted.
+// A float distance has a relative error below 4e-7, so the first six are the exact
+// six unless the seventh lies within 2e-6 of the sixth.
+struct Near7 {
+    float d[7];
+    int j[7];
+};
+
+__device__ __forceinline__ void near7_offer(Near7 &b, float4 q, const float xq[3], int j) {
+    const float fx = q.x - xq[0], fy = q.y - xq[1], fz = q.z - xq[2];
+    const float dv = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
+    if (!(dv < b.d[6])) return;
+#pragma unroll
+    for (int s = 6; s >= 1; --s) {
+        const bool in = dv < b.d[s], before = dv < b.d[s - 1];
+        b.j[s] = before ? b.j[s - 1] : (in ? j : b.j[s]);
+        b.d[s] = before ? b.d[s - 1] : (in ? dv : b.d[s]);
+    }
+    if (dv < b.d[0]) {
+        b.d[0] = dv;
+        b.j[0] = j;
+    }
+}
+
+// Returns 0 when every lane has its exact six, 1 when float distances cannot tell
+// some lane's sixth, 2 when the candidate list or the walk's stack would overflow.
+__device__ __forceinline__ int tile_near7(const Index &ix, int g, int i, bool live, const float xq[3], Near7 &b,
+                                           int *stk, int *cand) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int s = 0; s < 7; ++s) {
+        b.d[s] = INFINITY;
+        b.j[s] = -1;
+    }
+    const int i0 = 32 * g;
+    const float4 mine = live ? __ldg(ix.pts + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k = 1; k < 32; ++k) {   // the tile's own points, nearest in Morton order first
+        const int off = (k & 1) ? (k + 1) >> 1 : -(k >> 1);   // +1, -1, +2, -2, ..., -15, +16
+        const int t = (lane + off) & 31;
+        float4 q;
+        q.x = __shfl_sync(FULL, mine.x, t);
+        q.y = __shfl_sync(FULL, mine.y, t);
+        q.z = __shfl_sync(FULL, mine.z, t);
+        if (live && i0 + t < ix.n) near7_offer(b, q, xq, i0 + t);
+    }
+    float R = live ? b.d[5] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) R = fmaxf(R, __shfl_xor_sync(FULL, R, o));
+    if (!(R < INFINITY)) return 2;
+    const int nc = tile_candidates(ix, g, R, stk, cand);
+    if (nc < 0) return 2;
+    const float zero[3] = {0.0f, 0.0f, 0.0f};
+    for (int k = 0; k < nc; ++k) {
+        const int c = cand[k];
+        const bool need = live && obb_d2(obb_at(ix.obb, c - ix.L + ix.leaf0), xq, zero) * kObbShrink <= b.d[5];
+        if (!__any_sync(FULL, need)) continue;
+        const int beg = (c - ix.L) * kLeaf;
+        const int end = min(beg + kLeaf, ix.n);
+        if (need)
+            for (int j = beg; j < end; ++j) near7_offer(b, __ldg(ix.pts + j), xq, j);
+    }
+    return __any_sync(FULL, live && !(b.d[6] > b.d[5] * kTieWindow && b.d[5] < INFINITY)) ? 1 : 0;
+}
+
+// Sort of six non-negative doubles by their bits (they order alike).
+__device__ __forceinline__ void sort6(long long (&v)[6]) {
+    constexpr int A[12] = {0, 1, 2, 1, 3, 0, 2, 0, 2, 4, 1, 3}, B[12] = {5, 3, 4, 2, 4, 3, 5, 1, 3, 5, 2, 4};
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const long long x = v[A[k]], y = v[B[k]];
+        v[A[k]] = x < y ? x : y;
+        v[B[k]] = x < y ? y : x;
+    }
+}
+
+// write_knn6_stats for six neighbours in any order.
+__device__ __forceinline__ void write_near6_stats(const Index &ix, int i, const float xq[3], const Near7 &b,
+                                                  double *stat_d, double *stat_h) {
+    const double x0 = xq[0], x1 = xq[1], x2 = xq[2];
+    float4 ni = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (stat_h != nullptr) ni = ix.nrm[i];
+    long long dk[6], hk[6];
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        const float4 q = __ldg(ix.pts + b.j[s]);
+        const double a0 = (double)q.x - x0, a1 = (double)q.y - x1, a2 = (double)q.z - x2;
+        dk[s] = __double_as_longlong(a0 * a0 + a1 * a1 + a2 * a2);
+        hk[s] = __double_as_longlong(fabs(a0 * ni.x + a1 * ni.y + a2 * ni.z));
+    }
+    sort6(dk);
+    stat_d[i] = 0.5 * (sqrt(__longlong_as_double(dk[2])) + sqrt(__longlong_as_double(dk[3])));
+    if (stat_h != nullptr) {
+        sort6(hk);
+        stat_h[i] = 0.5 * (__longlong_as_double(hk[2]) + __longlong_as_double(hk[3]));
+    }
+}
+
+// Tiles whose candidate list does not fit (a scattered tile: its 32 points lie on
+// both sides of a gap of the Morton order) are left to k_knn6_rest: `rest` holds
+// their numbers, rest[-1] how many.
 __global__ void __launch_bounds__(kKnnBlock) k_knn6_tile(Index ix, double *__restrict__ stat_d,
-                                                         double *__restrict__ stat_h, int *__restrict__ overflow) {
+                                                         double *__restrict__ stat_h, int *__restrict__ rest) {
     __shared__ int s_stk[kKnnBlock / 32][kWarpStack];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int wpb = kKnnBlock / 32;
-    const int ngroups = (ix.n + 31) / 32;
+    const int g = blockIdx.x * (kKnnBlock / 32) + w;
+    if (g >= (ix.n + 31) / 32) return;
     int *stk = s_stk[w];
     int *cand = s_stk[w] + (kWarpStack - kKnnCand);
-    for (int g = blockIdx.x * wpb + w; g < ngroups; g += gridDim.x * wpb) {
-        const int i = 32 * g + lane;
-        const bool live = i < ix.n;
-        float xq[3] = {0.0f, 0.0f, 0.0f};
-        if (live) {
-            const float4 qi = __ldg(ix.pts + i);
-            xq[0] = qi.x;
-            xq[1] = qi.y;
-            xq[2] = qi.z;
-        }
+    const int i = 32 * g + lane;
+    const bool live = i < ix.n;
+    float xq[3] = {0.0f, 0.0f, 0.0f};
+    if (live) {
+        const float4 qi = __ldg(ix.pts + i);
+        xq[0] = qi.x;
+        xq[1] = qi.y;
+        xq[2] = qi.z;
+    }
+    Near7 nb;
+    const int rc = tile_near7(ix, g, i, live, xq, nb, stk, cand);
+    if (rc == 0) {
+        if (live) write_near6_stats(ix, i, xq, nb, stat_d, stat_h);
+        return;
+    }
+    __syncwarp();
+    if (rc == 1) {   // ties: FP64 distances
         Best6 b;
         if (tile_knn6(ix, g, i, live, xq, b, stk, cand)) {
             if (live) write_knn6_stats(ix, i, xq, b, stat_d, stat_h);
+            return;
+        }
+    }
+    if (lane == 0) rest[atomicAdd(rest - 1, 1)] = g;
+}
+
+// The points of the tiles k_knn6_tile left over, one per warp: by float distance
+// (near_knn), again in FP64 where that cannot tell the sixth.
+__global__ void __launch_bounds__(kKnnBlock) k_knn6_rest(Index ix, double *__restrict__ stat_d,
+                                                         double *__restrict__ stat_h, const int *__restrict__ rest,
+                                                         int *__restrict__ overflow) {
+    __shared__ int s_stk[kKnnBlock / 32][kWarpStack];
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t total = 32 * (int64_t)__ldg(rest - 1);
+    for (int64_t u = (int64_t)blockIdx.x * (kKnnBlock / 32) + w; u < total; u += (int64_t)gridDim.x * (kKnnBlock / 32)) {
+        const int i = 32 * __ldg(rest + (u >> 5)) + (int)(u & 31);
+        if (i >= ix.n) continue;   // uniform in the warp
+        const float4 qi = __ldg(ix.pts + i);
+        const float xq[3] = {qi.x, qi.y, qi.z};
+        NearK t;
+        const int rc = near_knn(ix, i, xq, i, 6, t, s_stk[w]);
+        __syncwarp();
+        if (rc != 0) {
+            Best6 b;
+            if (!warp_knn6(ix, i, xq, b, s_stk[w])) {
+                if (lane == 0) *overflow = 1;
+            } else if (lane == 0) {
+                write_knn6_stats(ix, i, xq, b, stat_d, stat_h);
+            }
+            __syncwarp();
             continue;
         }
-        __syncwarp();
-        for (int t = 0; t < 32 && 32 * g + t < ix.n; ++t) {   // point by point
-            const int it = 32 * g + t;
-            const float4 qt = __ldg(ix.pts + it);
-            const float xt[3] = {qt.x, qt.y, qt.z};
-            Best6 bt;
-            if (!warp_knn6(ix, it, xt, bt, stk)) {
-                if (lane == 0) *overflow = 1;
-                continue;
+        // one neighbour per lane; the 3rd and 4th smallest by rank
+        long long dk = 0, hk = 0;
+        if (lane < 6) {
+            const float4 q = __ldg(ix.pts + t.j);
+            const double a0 = (double)q.x - (double)xq[0], a1 = (double)q.y - (double)xq[1],
+                         a2 = (double)q.z - (double)xq[2];
+            dk = __double_as_longlong(a0 * a0 + a1 * a1 + a2 * a2);
+            if (stat_h != nullptr) {
+                const float4 ni = __ldg(ix.nrm + i);
+                hk = __double_as_longlong(fabs(a0 * ni.x + a1 * ni.y + a2 * ni.z));
             }
-            if (lane == 0) write_knn6_stats(ix, it, xt, bt, stat_d, stat_h);
-            __syncwarp();
+        }
+        int rd = 0, rh = 0;
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+            const long long od = __shfl_sync(FULL, dk, s), oh = __shfl_sync(FULL, hk, s);
+            rd += od < dk || (od == dk && s < lane);
+            rh += oh < hk || (oh == hk && s < lane);
+        }
+        const unsigned d2 = __ballot_sync(FULL, lane < 6 && rd == 2), d3 = __ballot_sync(FULL, lane < 6 && rd == 3);
+        const unsigned h2 = __ballot_sync(FULL, lane < 6 && rh == 2), h3 = __ballot_sync(FULL, lane < 6 && rh == 3);
+        const double v2 = __longlong_as_double(__shfl_sync(FULL, dk, __ffs(d2) - 1));
+        const double v3 = __longlong_as_double(__shfl_sync(FULL, dk, __ffs(d3) - 1));
+        const double u2 = __longlong_as_double(__shfl_sync(FULL, hk, __ffs(h2) - 1));
+        const double u3 = __longlong_as_double(__shfl_sync(FULL, hk, __ffs(h3) - 1));
+        if (lane == 0) {
+            stat_d[i] = 0.5 * (sqrt(v2) + sqrt(v3));
+            if (stat_h != nullptr) stat_h[i] = 0.5 * (u2 + u3);
         }
     }
 }
@@ -910,153 +1226,6 @@ __device__ __noinline__ bool warp_knn_k(const Index &ix, int i, const float xq[3
     return true;
 }
 
-// The 32 nearest points of a query by float distance, lane s the s-th.
-struct NearK {
-    float d;
-    int j;
-    float bound;   // the K-th distance
-    float spill;   // smallest distance that left the list
-};
-
-// Compare-exchange with lane ^ s, the smaller distance to the lower lane when
-// `up`. Equal distances stay where they are, in both lanes.
-__device__ __forceinline__ void near_exchange(float &d, int &j, int s, bool up) {
-    const unsigned FULL = 0xffffffffu;
-    const float od = __shfl_xor_sync(FULL, d, s);
-    const int oj = __shfl_xor_sync(FULL, j, s);
-    const bool keep_min = ((threadIdx.x & s) == 0) == up;
-    if (keep_min ? od < d : od > d) {
-        d = od;
-        j = oj;
-    }
-}
-
-__device__ __forceinline__ void near_scan(const Index &ix, const float xq[3], NearK &t, int K, int na, int nb,
-                                          bool two) {
-    const unsigned FULL = 0xffffffffu;
-    const float INF = __int_as_float(0x7f800000);
-    const int lane = threadIdx.x & 31;
-    float d = INF;
-    int j = -1;
-    if (lane < 16 || two) {
-        j = ((lane < 16 ? na : nb) - ix.L) * kLeaf + (lane & 15);
-        if (j < ix.n) {
-            const float4 q = __ldg(ix.pts + j);
-            const float fx = q.x - xq[0], fy = q.y - xq[1], fz = q.z - xq[2];
-            d = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
-            if (!(d * kShrink <= t.bound)) d = INF;
-        }
-    }
-    unsigned cm = __ballot_sync(FULL, d < INF);
-    if (cm == 0u) return;
-    if (__popc(cm) <= 3) {   // a few: insert one by one
-        while (cm) {
-            const int src = __ffs(cm) - 1;
-            cm &= cm - 1u;
-            const float dv = __shfl_sync(FULL, d, src);
-            const int jv = __shfl_sync(FULL, j, src);
-            const unsigned gm = __ballot_sync(FULL, t.d > dv);
-            const float ud = __shfl_up_sync(FULL, t.d, 1);
-            const int uj = __shfl_up_sync(FULL, t.j, 1);
-            t.spill = fminf(t.spill, gm == 0u ? dv : __shfl_sync(FULL, t.d, 31));
-            if (gm == 0u) continue;
-            const int pos = __ffs(gm) - 1;
-            if (lane >= pos) {
-                t.d = lane == pos ? dv : ud;
-                t.j = lane == pos ? jv : uj;
-            }
-        }
-    } else {   // sort the 32 descending, merge with the ascending list, keep the lower half
-#pragma unroll
-        for (int k = 2; k <= 32; k <<= 1)
-#pragma unroll
-            for (int o = k >> 1; o > 0; o >>= 1) near_exchange(d, j, o, (lane & k) != 0);
-        float out = t.d > d ? t.d : d;
-        if (d < t.d) {
-            t.d = d;
-            t.j = j;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) near_exchange(t.d, t.j, o, true);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) out = fminf(out, __shfl_xor_sync(FULL, out, o));
-        t.spill = fminf(t.spill, out);
-    }
-    t.bound = __shfl_sync(FULL, t.d, K - 1);
-}
-
-// The K nearest of point i in lanes 0 .. K-1. Returns 0 if they are the exact K,
-// 1 if float distances cannot tell, 2 if the stack would overflow.
-__device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3], int K, NearK &t, int *stk) {
-    const unsigned FULL = 0xffffffffu;
-    const float INF = __int_as_float(0x7f800000);
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    const float zero[3] = {0.0f, 0.0f, 0.0f};
-    t.d = t.bound = t.spill = INF;
-    t.j = -1;
-    const int depth = 31 - __clz(ix.L);
-    const int start = ix.L + i / kLeaf;
-    near_scan(ix, xq, t, K, start, start ^ 1, depth > 0);   // the point's bucket and its sibling first
-    int sp;
-    {
-        int c = 0;
-        bool pass = false;
-        if (lane < depth - 1) {
-            c = (start >> (depth - 1 - lane)) ^ 1;
-            pass = box_d2(__ldg(ix.nodes + 2 * c), __ldg(ix.nodes + 2 * c + 1), xq, zero) * kShrink <= t.bound;
-        }
-        const unsigned m = __ballot_sync(FULL, pass);
-        if (pass) stk[__popc(m & below)] = c;
-        sp = __popc(m);
-    }
-    __syncwarp();
-    while (sp > 0) {
-        const int k = min(32, sp);
-        const int node = (lane < k) ? stk[sp - 1 - lane] : 0;
-        sp -= k;
-        __syncwarp();
-        // inner nodes at least two levels above the buckets expand to four grandchildren, others to two children
-        int c0 = 0, nc = 0;
-        bool leaf_ok = false;
-        if (node != 0) {
-            if (node < ix.L) {
-                const bool deep = 2 * node < ix.L;
-                c0 = deep ? 4 * node : 2 * node;
-                nc = deep ? 4 : 2;
-            } else {
-                leaf_ok = box_d2(__ldg(ix.nodes + 2 * node), __ldg(ix.nodes + 2 * node + 1), xq, zero) * kShrink
-                              <= t.bound &&
-                          obb_d2(obb_at(ix.obb, node - ix.L + ix.leaf0), xq, zero) * kObbShrink <= t.bound;
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            bool ok = false;
-            if (g < nc)
-                ok = box_d2(__ldg(ix.nodes + 2 * (c0 + g)), __ldg(ix.nodes + 2 * (c0 + g) + 1), xq, zero) * kShrink <=
-                     t.bound;
-            const unsigned mg = __ballot_sync(FULL, ok);
-            if (sp + __popc(mg) > kWarpStack) return 2;
-            if (ok) stk[sp + __popc(mg & below)] = c0 + g;
-            sp += __popc(mg);
-        }
-        unsigned lm = __ballot_sync(FULL, leaf_ok);
-        while (lm) {   // two buckets per pass: lanes 0-15 and 16-31
-            const int la = __ffs(lm) - 1;
-            lm &= lm - 1u;
-            const bool two = lm != 0u;
-            const int lb = two ? __ffs(lm) - 1 : la;
-            if (two) lm &= lm - 1u;
-            const int na = __shfl_sync(FULL, node, la), nb = __shfl_sync(FULL, node, lb);
-            near_scan(ix, xq, t, K, na, nb, two);
-        }
-        __syncwarp();
-    }
-    const float next = K < 32 ? __shfl_sync(FULL, t.d, K & 31) : t.spill;
-    return !(t.bound < INF) || (next <= t.bound * kTieWindow && next < INF) ? 1 : 0;   // not finite: distances beyond float
-}
-
 // Eigenvector of the smallest eigenvalue of the symmetric matrix e (xx, xy, xz,
 // yy, yz, zz) by cyclic Jacobi rotations in FP64.
 __device__ __noinline__ void jacobi_axis(const double e[6], double n[3]) {
@@ -1161,7 +1330,7 @@ __global__ void __launch_bounds__(kKnnBlock) k_normals(Index ix, int K, int per_
         const float4 qi = __ldg(ix.pts + i);
         const float xq[3] = {qi.x, qi.y, qi.z};
         NearK t;
-        int rc = near_knn(ix, (int)i, xq, K, t, s_stk[w]);
+        int rc = near_knn(ix, (int)i, xq, -1, K, t, s_stk[w]);
         __syncwarp();
         if (rc == 1) {
             TopK e;
@@ -1212,38 +1381,48 @@ __global__ void __launch_bounds__(kKnnBlock) k_normals(Index ix, int K, int per_
 // Grid-wide form of block_median_pair for large n (the nu_min medians of a
 // whole target): the same eight 8-bit radix passes over the IEEE bit patterns,
 // but each pass's two histograms are built by every block (shared-memory
-// histograms folded into MedianState::hist with one atomic per bin and block)
-// and one block then locates each rank's bin. Counts do not depend on the
+// histograms folded into MedianState::hist with one atomic per bin and block). Counts do not depend on the
 // order of the atomics, so the result is the one block_median_pair gives.
+// One launch per radix pass: the last block to fold its histograms locates each
+// rank's bin and clears the histograms for the next pass. Two arrays of n values
+// (the point and the plane statistic) are taken side by side, blockIdx.y each
+// (500,000 points, both statistics: 34 launches 162 us, 9 launches 86 us).
 // Launch order: k_median_init, then for shift = 56, 48, ..., 0 one
-// k_median_hist and one k_median_pick (64 threads); the last pick writes
-// 0.5 * (lo + hi) to *out.
+// k_median_pass; the last writes 0.5 * (lo + hi) to out[blockIdx.y].
 struct MedianState {
     unsigned long long prefix[2];
     int k[2];
+    unsigned int done;   // blocks that folded their histograms in this pass
+    unsigned int pad;
     unsigned int hist[2][256];
 };
 
 __global__ void k_median_init(MedianState *st, int n) {
+    st += blockIdx.x;
     for (int b = threadIdx.x; b < 512; b += blockDim.x) (&st->hist[0][0])[b] = 0u;
     if (threadIdx.x == 0) {
         st->prefix[0] = st->prefix[1] = 0ull;
         st->k[0] = (n - 1) / 2;
         st->k[1] = n / 2;
+        st->done = 0u;
     }
 }
 
-__global__ void k_median_hist(const double *v, int n, MedianState *st, int shift) {
+__global__ void __launch_bounds__(256) k_median_pass(const double *v0, const double *v1, int n, MedianState *st,
+                                                     int shift, double *out) {
     __shared__ unsigned int hist[2][256];
+    __shared__ bool s_last;
     const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double *v = blockIdx.y ? v1 : v0;
+    st += blockIdx.y;
     for (int b = threadIdx.x; b < 512; b += blockDim.x) (&hist[0][0])[b] = 0u;
     __syncthreads();
     const unsigned long long p0 = st->prefix[0], p1 = st->prefix[1];
     const unsigned long long mask = (shift == 56) ? 0ull : (~0ull << (shift + 8));
     // every lane runs every round (the peer match is warp-wide)
-    for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
-        const int i = base + threadIdx.x;
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = base + threadIdx.x;
         unsigned long long key = ~0ull;
         if (i < n) key = (unsigned long long)__double_as_longlong(__ldcg(v + i));
         const int bin = (int)((key >> shift) & 255ull);
@@ -1259,16 +1438,17 @@ __global__ void k_median_hist(const double *v, int n, MedianState *st, int shift
         const unsigned c = (&hist[0][0])[b];
         if (c) atomicAdd(&st->hist[0][0] + b, c);
     }
-}
-
-__global__ void __launch_bounds__(64) k_median_pick(MedianState *st, int shift, double *out) {
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
     if (w < 2) {   // warp r finds the bin holding its rank (as block_median_pair)
         unsigned c[8], sum = 0;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            c[q] = st->hist[w][8 * lane + q];
+            c[q] = __ldcg(&st->hist[w][8 * lane + q]);
             sum += c[q];
         }
         unsigned incl = sum;
@@ -1293,8 +1473,12 @@ __global__ void __launch_bounds__(64) k_median_pick(MedianState *st, int shift, 
     }
     __syncthreads();
     for (int b = threadIdx.x; b < 512; b += blockDim.x) (&st->hist[0][0])[b] = 0u;   // for the next pass
-    if (shift == 0 && threadIdx.x == 0)
-        *out = 0.5 * (__longlong_as_double((long long)st->prefix[0]) + __longlong_as_double((long long)st->prefix[1]));
+    if (threadIdx.x == 0) {
+        st->done = 0u;
+        if (shift == 0)
+            out[blockIdx.y] =
+                0.5 * (__longlong_as_double((long long)st->prefix[0]) + __longlong_as_double((long long)st->prefix[1]));
+    }
 }
 
 struct BoxResult {
@@ -1491,19 +1675,18 @@ cudaError_t build_fp16_storage(TargetDev *t, cudaStream_t s) {
     return cudaSuccess;
 }
 
-cudaError_t launch_median(const double *v, int n, void *scratch, double *out_dev, cudaStream_t s) {
-    static_assert(sizeof(MedianState) <= (size_t)kMedianScratchBytes, "median scratch");
+cudaError_t launch_median(const double *v, const double *v2, int n, void *scratch, double *out_dev, cudaStream_t s) {
+    static_assert(2 * sizeof(MedianState) <= (size_t)kMedianScratchBytes, "median scratch");
     MedianState *mst = static_cast<MedianState *>(scratch);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int arrays = v2 != nullptr ? 2 : 1;
     const unsigned mblocks = (unsigned)std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)(sms > 0 ? sms : 152) * 4);
-    k_median_init<<<1, 256, 0, s>>>(mst, n);
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        k_median_hist<<<mblocks, 256, 0, s>>>(v, n, mst, shift);
-        k_median_pick<<<1, 64, 0, s>>>(mst, shift, out_dev);
-    }
-    counters().launches += 17;
+    k_median_init<<<arrays, 256, 0, s>>>(mst, n);
+    for (int shift = 56; shift >= 0; shift -= 8)
+        k_median_pass<<<dim3(mblocks, arrays), 256, 0, s>>>(v, v2, n, mst, shift, out_dev);
+    counters().launches += 9;
     return cudaGetLastError();
 }
 
@@ -1515,9 +1698,9 @@ cudaError_t target_nu_stats(TargetDev *t, cudaStream_t s) {
         return cudaSuccess;
     }
     double *sd = nullptr, *sh = nullptr, *out = nullptr;
-    MedianState *mst = nullptr;
+    void *mst = nullptr;
     cudaError_t e = pool_alloc(&sd, sizeof(double) * t->n, s);
-    if (e == cudaSuccess) e = pool_alloc(&mst, sizeof(MedianState), s);
+    if (e == cudaSuccess) e = pool_alloc(&mst, kMedianScratchBytes, s);
     if (e == cudaSuccess && t->has_normals) e = pool_alloc(&sh, sizeof(double) * t->n, s);
     if (e == cudaSuccess) e = pool_alloc(&out, 3 * sizeof(double), s);
     int *flag = reinterpret_cast<int *>(out + 2);
@@ -1531,15 +1714,21 @@ cudaError_t target_nu_stats(TargetDev *t, cudaStream_t s) {
                                                  (int64_t)(sms > 0 ? sms : 152) * 16);
         if (t->L >= 4) {
             const int64_t tiles = (t->n + 31) / 32;
-            const int64_t tblocks = std::min<int64_t>((tiles + kKnnBlock / 32 - 1) / (kKnnBlock / 32),
-                                                      (int64_t)(sms > 0 ? sms : 152) * 16);
-            k_knn6_tile<<<(unsigned)tblocks, kKnnBlock, 0, s>>>(ix, sd, sh, flag);
+            int *rest = nullptr;
+            e = pool_alloc(&rest, sizeof(int) * (size_t)(tiles + 1), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(rest, 0, sizeof(int), s);
+            if (e == cudaSuccess) {
+                k_knn6_tile<<<(unsigned)((tiles + kKnnBlock / 32 - 1) / (kKnnBlock / 32)), kKnnBlock, 0, s>>>(
+                    ix, sd, sh, rest + 1);
+                k_knn6_rest<<<(sms > 0 ? sms : 152) * 8, kKnnBlock, 0, s>>>(ix, sd, sh, rest + 1, flag);
+                counters().launches += 1;
+            }
+            if (rest) cudaFreeAsync(rest, s);
         } else {
             k_knn6_stats<<<(unsigned)blocks, kKnnBlock, 0, s>>>(ix, sd, sh, flag);
         }
         counters().launches += 1;
-        for (int which = 0; which < (sh ? 2 : 1); ++which)
-            if (e == cudaSuccess) e = launch_median(which ? sh : sd, (int)t->n, mst, out + which, s);
+        if (e == cudaSuccess) e = launch_median(sd, sh, (int)t->n, mst, out, s);
         double h[3] = {0.0, 0.0, 0.0};
         if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, s);
         counters().d2h += 3 * sizeof(double);
