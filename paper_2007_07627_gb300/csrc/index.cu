@@ -47,9 +47,13 @@ __global__ void k_box_partial(const float *__restrict__ x, const float *__restri
             sm[a] += (double)v;
         }
         if (nrm != nullptr) {
-            const double a0 = nrm[3 * i], a1 = nrm[3 * i + 1], a2 = nrm[3 * i + 2];
-            const double l2 = a0 * a0 + a1 * a1 + a2 * a2;
-            if (!(fabs(l2 - 1.0) <= 2e-3) && !(zero_normals_ok && l2 == 0.0)) bad = 1;
+            const float n0 = nrm[3 * i], n1 = nrm[3 * i + 1], n2 = nrm[3 * i + 2];
+            const float lf = fmaf(n2, n2, fmaf(n1, n1, n0 * n0));
+            if (!(fabsf(lf - 1.0f) <= 1.999e-3f)) {   // not clearly unit (float: exact to 3e-7): the FP64 test decides
+                const double a0 = n0, a1 = n1, a2 = n2;
+                const double l2 = a0 * a0 + a1 * a1 + a2 * a2;
+                if (!(fabs(l2 - 1.0) <= 2e-3) && !(zero_normals_ok && l2 == 0.0)) bad = 1;
+            }
         }
     }
     __syncthreads();
@@ -158,21 +162,58 @@ __global__ void k_gather(const float *__restrict__ x, const float *__restrict__ 
         nout[i] = make_float4(nrm[3 * (int64_t)o], nrm[3 * (int64_t)o + 1], nrm[3 * (int64_t)o + 2], 0.0f);
 }
 
-__global__ void k_leaf_boxes(const float4 *__restrict__ pts, int64_t n, int L, float4 *__restrict__ nodes) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= L) return;
+// Axis-aligned boxes of the tree, 256 nodes of a level per block and the levels
+// above them up to eight: the bucket level (LEAF) from the points, a higher one
+// from the boxes written by the launch before. One launch per eight levels (a
+// launch per level, 15 of them, took 42 us for 500,000 points).
+template <bool LEAF>
+__global__ void __launch_bounds__(256) k_boxes(const float4 *__restrict__ pts, int64_t n, int size,
+                                               float4 *__restrict__ nodes) {
+    __shared__ float4 s_lo[256], s_hi[256];
+    const int t = threadIdx.x;
+    const int l = blockIdx.x * 256 + t;
     float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.0f);
     float4 hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.0f);
-    const int64_t beg = (int64_t)l * kLeaf;
-    const int64_t end = beg + kLeaf < n ? beg + kLeaf : n;
-    for (int64_t j = beg; j < end; ++j) {
-        const float4 p = pts[j];
-        lo.x = fminf(lo.x, p.x); lo.y = fminf(lo.y, p.y); lo.z = fminf(lo.z, p.z);
-        hi.x = fmaxf(hi.x, p.x); hi.y = fmaxf(hi.y, p.y); hi.z = fmaxf(hi.z, p.z);
+    if (l < size) {
+        const int64_t node = (int64_t)size + l;
+        if (LEAF) {
+            const int64_t beg = (int64_t)l * kLeaf;
+            const int64_t end = beg + kLeaf < n ? beg + kLeaf : n;
+            for (int64_t j = beg; j < end; ++j) {
+                const float4 p = pts[j];
+                lo.x = fminf(lo.x, p.x); lo.y = fminf(lo.y, p.y); lo.z = fminf(lo.z, p.z);
+                hi.x = fmaxf(hi.x, p.x); hi.y = fmaxf(hi.y, p.y); hi.z = fmaxf(hi.z, p.z);
+            }
+            nodes[2 * node] = lo;
+            nodes[2 * node + 1] = hi;
+        } else {
+            lo = nodes[2 * node];
+            hi = nodes[2 * node + 1];
+        }
     }
-    const int node = L + l;
-    nodes[2 * node] = lo;
-    nodes[2 * node + 1] = hi;
+    s_lo[t] = lo;
+    s_hi[t] = hi;
+    __syncthreads();
+    int level = size, first = blockIdx.x * 256;   // nodes of the level, and this block's first
+    for (int cnt = 128; cnt >= 1 && level > 1; cnt >>= 1) {
+        level >>= 1;
+        first >>= 1;
+        if (t < cnt) {
+            const float4 a0 = s_lo[2 * t], a1 = s_hi[2 * t], b0 = s_lo[2 * t + 1], b1 = s_hi[2 * t + 1];
+            lo = make_float4(fminf(a0.x, b0.x), fminf(a0.y, b0.y), fminf(a0.z, b0.z), 0.0f);
+            hi = make_float4(fmaxf(a1.x, b1.x), fmaxf(a1.y, b1.y), fmaxf(a1.z, b1.z), 0.0f);
+            if (first + t < level) {
+                nodes[2 * ((int64_t)level + first + t)] = lo;
+                nodes[2 * ((int64_t)level + first + t) + 1] = hi;
+            }
+        }
+        __syncthreads();
+        if (t < cnt) {
+            s_lo[t] = lo;
+            s_hi[t] = hi;
+        }
+        __syncthreads();
+    }
 }
 
 // Box of no points: farther than any finite bound.
@@ -201,9 +242,8 @@ __global__ void k_leaf_obb(const float4 *__restrict__ pts, int64_t n, int L, flo
 
 // Oriented boxes of the patches three, six and nine levels above the buckets (128,
 // 1,024 and 8,192 points), one per NT threads: axes of the points' scatter about the
-// axis-aligned box's middle, extents in float about a float centre. The float
-// rounding of the extents (5.2e-7 of the radius, as in obb_eval) is inside the
-// widening, twice obb_fit's. `shift` = 3, 6 or 9.
+// axis-aligned box's middle, extents about a float centre, widened as obb_fit's.
+// `shift` = 3, 6 or 9.
 template <int NT>
 __global__ void __launch_bounds__(256) k_patch_obb(const float4 *__restrict__ pts, int64_t n, int L, int shift,
                                                    const float4 *__restrict__ nodes, float4 *__restrict__ obb) {
@@ -262,11 +302,8 @@ __global__ void __launch_bounds__(256) k_patch_obb(const float4 *__restrict__ pt
     const float xy = v[4] - v[0] * v[1] * ic, xz = v[5] - v[0] * v[2] * ic, yz = v[7] - v[1] * v[2] * ic;
     float A[3][3] = {{v[3] - v[0] * v[0] * ic, xy, xz}, {xy, v[6] - v[1] * v[1] * ic, yz},
                      {xz, yz, v[8] - v[2] * v[2] * ic}};
-    double ax[3][3];
-    obb_axes(A, ax);
     float a[3][3];
-    for (int k = 0; k < 3; ++k)
-        for (int r = 0; r < 3; ++r) a[k][r] = (float)ax[k][r];
+    obb_axes(A, a);
     float e[6] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max u, max -u
     for (int k = tid; k < cnt; k += NT) {
         const float4 p = pts[beg + k];
@@ -296,7 +333,7 @@ __global__ void __launch_bounds__(256) k_patch_obb(const float4 *__restrict__ pt
         return;
     }
     const float r = sqrtf(h[3]) * (1.0f + 1e-6f);
-    for (int k = 0; k < 3; ++k) h[k] = f32_round_up(h[k] * (1.0 + 2e-6) + 4e-6 * r + 1e-37);
+    for (int k = 0; k < 3; ++k) h[k] = obb_widen(h[k], r);
     o[0] = make_float4(c[0], c[1], c[2], h[0]);
     for (int k = 0; k < 3; ++k) o[8 + 8 * k] = make_float4(a[k][0], a[k][1], a[k][2], k == 0 ? h[1] : (k == 1 ? h[2] : r));
 }
@@ -329,15 +366,6 @@ __global__ void k_level_obb(const float4 *__restrict__ nodes, int L, int size, i
     o[8] = make_float4(1.0f, 0.0f, 0.0f, h[1]);
     o[16] = make_float4(0.0f, 1.0f, 0.0f, h[2]);
     o[24] = make_float4(0.0f, 0.0f, 1.0f, f32_round_up(r));
-}
-
-__global__ void k_level_boxes(float4 *__restrict__ nodes, int first, int count) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    const int i = first + k;
-    const float4 a0 = nodes[4 * i], a1 = nodes[4 * i + 1], b0 = nodes[4 * i + 2], b1 = nodes[4 * i + 3];
-    nodes[2 * i] = make_float4(fminf(a0.x, b0.x), fminf(a0.y, b0.y), fminf(a0.z, b0.z), 0.0f);
-    nodes[2 * i + 1] = make_float4(fmaxf(a1.x, b1.x), fmaxf(a1.y, b1.y), fmaxf(a1.z, b1.z), 0.0f);
 }
 
 // Six nearest target points of every target point, the point itself excluded
@@ -1610,11 +1638,11 @@ cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cuda
     if (e == cudaSuccess) {
         t->obb = t->nodes + 4 * (size_t)L;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q_dev, n_dev, order, n, t->pts, t->nrm);
-        k_leaf_boxes<<<(L + 255) / 256, 256, 0, s>>>(t->pts, n, L, t->nodes);
+        k_boxes<true><<<(L + 255) / 256, 256, 0, s>>>(t->pts, n, L, t->nodes);
         k_leaf_obb<<<(L + 127) / 128, 128, 0, s>>>(t->pts, n, L, t->obb);
         counters().launches += 3;
-        for (int first = L / 2; first >= 1; first /= 2) {
-            k_level_boxes<<<(first + 255) / 256, 256, 0, s>>>(t->nodes, first, first);
+        for (int size = L / 256; size > 1; size /= 256) {
+            k_boxes<false><<<(size + 255) / 256, 256, 0, s>>>(t->pts, n, size, t->nodes);
             counters().launches += 1;
         }
         const int first = wide_first(L);
