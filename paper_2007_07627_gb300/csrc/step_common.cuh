@@ -47,7 +47,7 @@ __device__ __forceinline__ void block_reduce_store(double (&acc)[K], double *out
 
 // Fixed-order reduction of the tile records: thread t < G K (G = kBlock / K row
 // groups) sums column t mod K over rows g, g + G, g + 2 G, ... (g = t / K) in
-// order, eight loads in flight; the G partial sums of a column are then added
+// order, sixteen loads in flight; the G partial sums of a column are then added
 // in group order. `red` holds kBlock doubles of shared memory.
 template <int K>
 __device__ __forceinline__ void reduce_tiles(const double *partial, int ntiles, double *S, double *red) {
@@ -57,14 +57,29 @@ __device__ __forceinline__ void reduce_tiles(const double *partial, int ntiles, 
         const int k = t % K, g = t / K;
         double v = 0.0;
         int r = g;
-        for (; r + G * 7 < ntiles; r += G * 8) {
-            double x[8];
+        double x[8];
+        if (r + G * 7 < ntiles) {   // the next batch is loaded before this one is added
 #pragma unroll
             for (int u = 0; u < 8; ++u) x[u] = __ldcg(partial + (size_t)(r + G * u) * K + k);
+            for (r += G * 8; r + G * 7 < ntiles; r += G * 8) {
+                double y[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) y[u] = __ldcg(partial + (size_t)(r + G * u) * K + k);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v += x[u];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = y[u];
+            }
 #pragma unroll
             for (int u = 0; u < 8; ++u) v += x[u];
         }
-        for (; r < ntiles; r += G) v += __ldcg(partial + (size_t)r * K + k);
+        // the rest, fewer than eight rows, loaded together
+#pragma unroll
+        for (int u = 0; u < 7; ++u)
+            if (r + G * u < ntiles) x[u] = __ldcg(partial + (size_t)(r + G * u) * K + k);
+#pragma unroll
+        for (int u = 0; u < 7; ++u)
+            if (r + G * u < ntiles) v += x[u];
         red[t] = v;
     }
     __syncthreads();
