@@ -395,8 +395,9 @@ fricp_status register_impl(const fricp_target *t, const float *p_xyz, const floa
     DevBuf<float4> src;
     DevBuf<PairState> st_dev;
     DevBuf<double> partial, resid, trace_dev;
-    DevBuf<int> prev;
+    DevBuf<int> prev, hard;
     if (src.alloc(m, s) != cudaSuccess || st_dev.alloc(1, s) != cudaSuccess || prev.alloc(m, s) != cudaSuccess ||
+        hard.alloc(fricp::hard_ints(m), s) != cudaSuccess ||
         partial.alloc((size_t)ntiles * fricp::kMaxSums, s) != cudaSuccess ||
         resid.alloc(robust ? m : 1, s) != cudaSuccess || trace_dev.alloc(trace_capacity, s) != cudaSuccess)
         return fail(FRICP_ENOMEM, "device allocation for the registration");
@@ -435,6 +436,7 @@ fricp_status register_impl(const fricp_target *t, const float *p_xyz, const floa
     a.src = src.p;
     a.src_nrm = p_normals ? src_nrm.p : nullptr;
     a.prev = prev.p;
+    a.hard = hard.p;
     a.partial = partial.p;
     a.resid = resid.p;
     a.trace = trace_capacity > 0 ? trace_dev.p : nullptr;
@@ -442,7 +444,7 @@ fricp_status register_impl(const fricp_target *t, const float *p_xyz, const floa
     double pass_ms = 0.0, search_ms = 0.0;
     st = run_steps(a, prm.variant, ntiles, prm, s, st_dev.p, &leak, &pass_ms, &search_ms, h.init_median_ext ? m : 0);
     if (leak) {
-        src.leak = st_dev.leak = partial.leak = resid.leak = trace_dev.leak = prev.leak = rec.leak = src_nrm.leak = true;
+        src.leak = st_dev.leak = partial.leak = resid.leak = trace_dev.leak = prev.leak = hard.leak = rec.leak = src_nrm.leak = true;
         p.owned = nullptr;
     }
     if (st != FRICP_OK && st != FRICP_ETIMEOUT) return st;

@@ -186,12 +186,13 @@ __global__ void __launch_bounds__(kBlock, 4) k_nn_batch(const Slot *__restrict__
         for (int k = i0; k < i1; k += kGroupQ) {
             const int i = k + lane / kGroup;
             const bool live = i < i1;
+            int work = 0;
             if (h.prec == PREC_FP32)
-                seed = search_group<PREC_FP32>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed);
+                seed = search_group<PREC_FP32>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed, work);
             else if (h.prec == PREC_FP16)
-                seed = search_group<PREC_FP16>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed);
+                seed = search_group<PREC_FP16>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed, work);
             else
-                seed = search_group<PREC_FP64>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed);
+                seed = search_group<PREC_FP64>(sl.ix, sl.src, sl.prev, h, i, live, p2p, stk, seed, work);
         }
     }
 }

@@ -119,6 +119,7 @@ struct PairState {
     int capexit;            // the running line search started from a cap check
     int ls_l;
     int hlen;
+    int hard_n[2][2];       // hard tickets listed for the passes of either parity, by class (k_nn)
     int init_median_ext;    // the first pass leaves the nu_max median to the host's grid-wide select (k_after_init)
     double nu;
     double E_prev;
@@ -160,6 +161,7 @@ struct StepArgs {
     const float4 *src_nrm = nullptr;   // M source normals in the same order (symmetric objective), or null
     int *prev;             // M: correspondence (sorted target index) of the last pass, -1 if none;
                            //    the search kernel overwrites it with this pass's correspondence
+    int *hard = nullptr;   // hard_ints(M): lists and flags of the hard tickets (k_nn), or null: plain order
     double *partial;       // ntiles * kMaxSums
     double *resid;         // M per-point residuals (PH_INIT)
     double *trace;         // trace_cap energies
@@ -399,6 +401,10 @@ constexpr int kWarpStack = 1024;  // walk stack of a warp in the neighbour kerne
 constexpr int kGroup = 8;                         // lanes per query
 constexpr int kGroupQ = 32 / kGroup;              // queries per warp
 constexpr int kGroupC = 8 / kGroup;               // children per lane
+// Tickets of k_nn (kGroupQ queries each) over M queries, and the ints of their
+// lists and flags: per parity of the pass, a list of T tickets and T flag bytes.
+FRICP_HD inline int64_t search_tickets(int64_t M) { return (M + kGroupQ - 1) / kGroupQ; }
+FRICP_HD inline int64_t hard_ints(int64_t M) { return 2 * (search_tickets(M) + (search_tickets(M) + 3) / 4); }
 constexpr int kGroupDepth = 9;                    // inner levels of a tree over 2^30 points: ceil(26 / 3)
 constexpr int kGroupStack = 7 * kGroupDepth + 1;  // stack entries per group
 constexpr unsigned kGroupMask = (1u << kGroup) - 1u;
@@ -418,10 +424,11 @@ FRICP_HD inline int wide_child(int first, int p) { return 8 * p + 8 * first - 56
 
 // Walk the tree for the point x = xh + xl of this group, offering every point of
 // every bucket within `bound` to `offer(j, p)`, which returns the smallest float
-// distance this lane was offered so far.
+// distance this lane was offered so far. `work` counts the warp's rounds and bucket
+// scans.
 template <int PREC, class Offer>
 __device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], const float xl[3], float &bound,
-                                           float2 *stk, bool live, Offer offer) {
+                                           float2 *stk, bool live, int &work, Offer offer) {
     constexpr bool AABB = PREC == PREC_FP16;
     const unsigned FULL = 0xffffffffu;
     const float INF = __int_as_float(0x7f800000), OUT = __int_as_float(0x7fc00000);   // OUT: not within any bound
@@ -435,6 +442,7 @@ __device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], c
                                                   // positions begin with 8 - first empty boxes that must not be entered
     int sp = 0;
     while (__any_sync(FULL, cnt != 0)) {
+        ++work;
         const bool leaf = AABB ? base >= leaf0 : base + 7 >= leaf0;
         float key[kGroupC];
         unsigned near = 0xffffffffu;
@@ -469,6 +477,7 @@ __device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], c
         bool scan = any && leaf;
         while (__any_sync(FULL, scan)) {   // the nearest bucket, then the others that stay within the bound
             float d = INF;
+            ++work;
             if (scan) {
                 const int j0 = (base + w - leaf0) * kLeaf + gl;
 #pragma unroll
@@ -519,7 +528,7 @@ __device__ __forceinline__ void group_walk(const Index &ix, const float xh[3], c
 // two such points, by a second walk within the window.
 template <int PREC>
 __device__ __forceinline__ int group_nn(const Index &ix, const float xh[3], const float xl[3], float bound,
-                                        float2 *stk, bool live) {
+                                        float2 *stk, bool live, int &work) {
     const unsigned FULL = 0xffffffffu;
     const float INF = __int_as_float(0x7f800000);
     const int lane = threadIdx.x & 31;
@@ -527,7 +536,7 @@ __device__ __forceinline__ int group_nn(const Index &ix, const float xh[3], cons
     const float limit = PREC == PREC_FP64 ? bound * kTieWindow : bound;
     float d1 = INF, d2 = INF;
     int j1 = -1;
-    group_walk<PREC>(ix, xh, xl, bound, stk, live, [&](int j, float4 p) {
+    group_walk<PREC>(ix, xh, xl, bound, stk, live, work, [&](int j, float4 p) {
         const float d = point_d2f(xh, xl, p);
         d2 = fminf(d2, fmaxf(d1, d));
         if (d < d1) j1 = j;
@@ -552,7 +561,7 @@ __device__ __forceinline__ int group_nn(const Index &ix, const float xh[3], cons
         if (__any_sync(FULL, again)) {
             float bd = win;
             if (again) q.bestf = best;
-            group_walk<PREC>(ix, xh, xl, bd, stk, again, [&](int jj, float4 p) {
+            group_walk<PREC>(ix, xh, xl, bd, stk, again, work, [&](int jj, float4 p) {
                 nn_offer<PREC>(q, p, jj);
                 return win;
             });

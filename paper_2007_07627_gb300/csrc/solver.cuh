@@ -625,8 +625,10 @@ static __device__ __noinline__ void solver_step(Team tm, PairState *gst, const d
         }
     }
     set_head_cache(tm, st);
-    st->counter = 0u;   // the next pass's tile and search tickets start over
+    // the next pass's tickets start over (reset_tickets)
+    st->counter = 0u;
     st->nn_next = 0u;
+    st->hard_n[(st->device_steps + 1) & 1][0] = st->hard_n[(st->device_steps + 1) & 1][1] = 0;
     store_state(tm, st, gst);
 }
 

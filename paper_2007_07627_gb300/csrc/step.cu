@@ -17,6 +17,7 @@ namespace fricp {
 
 namespace {
 
+constexpr int kHardWork = 64;    // rounds and scans (24 on average) above which a ticket is hard, half of it: fairly hard
 constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket of a first pass
 
 // Search kernel: persistent warps take runs of Morton-adjacent queries, four
@@ -28,6 +29,13 @@ constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket
 // sixteen left the last tickets running alone: 335 us against 218 us, ellipsoids,
 // M = 200,000); a first pass takes longer runs, whose queries start from the
 // result of the one before.
+//
+// A few queries (outliers about equally far from a large part of the target) walk
+// ten times the average, and one that starts late runs on alone. They are the same
+// ones from pass to pass, so each pass lists its hard tickets for the next, which
+// takes them first. Every ticket is searched once either way. (Ellipsoids, M =
+// 200,000: 197 -> 157 us; field, M = 80,000: 91 -> 82 us; thresholds of 48, 96 and
+// 160: 158, 161, 169 us.)
 template <int PREC>
 __global__ void __launch_bounds__(kBlock) k_nn(StepArgs a) {
     __shared__ StepHead h;
@@ -39,21 +47,43 @@ __global__ void __launch_bounds__(kBlock) k_nn(StepArgs a) {
     const int lane = threadIdx.x & 31;
     float2 *stk = s_stk[threadIdx.x / kGroup];
     const unsigned warps = gridDim.x * (kBlock / 32);
-    const bool cold = a.st->device_steps == 0;
-    const int rounds = cold ? max(1, min(kColdRounds, (int)(h.M / (2 * kGroupQ * warps)))) : 1;
-    unsigned e = blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+    const int step = a.st->device_steps;
+    const int rounds = step == 0 ? max(1, min(kColdRounds, (int)(h.M / (2 * kGroupQ * warps)))) : 1;
+    // hard tickets listed by the pass before: class 0 from the front of its list, class 1 from the back
+    const int T = (int)search_tickets(h.M), par = step & 1;
+    const int n0 = a.hard ? a.st->hard_n[par][0] : 0, n1 = a.hard ? a.st->hard_n[par][1] : 0, nh = n0 + n1;
+    const int *list = a.hard + (size_t)par * T;
+    int *list_out = a.hard + (size_t)(par ^ 1) * T;
+    unsigned char *flags = reinterpret_cast<unsigned char *>(a.hard + 2 * (size_t)T);
+    const unsigned char *flag = flags + (size_t)par * T;
+    unsigned char *flag_out = flags + (size_t)(par ^ 1) * T;
+    unsigned u = blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
     for (;;) {
-        const long long i0 = (long long)e * (kGroupQ * rounds);
-        if (i0 >= h.M) break;
+        long long e;   // first ticket of this warp's run
+        if (u < (unsigned)nh)
+            e = u < (unsigned)n0 ? list[u] : list[T - 1 - (int)(u - n0)];
+        else
+            e = (long long)(u - nh) * rounds;
+        if (e >= T) break;
         unsigned nx = 0;
         if (lane == 0) nx = warps + atomicAdd(&a.st->nn_next, 1u);
-        int seed = -1;
-        for (int r = 0; r < rounds; ++r) {
-            const int i = (int)i0 + r * kGroupQ + lane / kGroup;
-            if (i - lane / kGroup >= h.M) break;
-            seed = search_group<PREC>(a.ix, a.src, a.prev, h, i, i < h.M, p2p, stk, seed);
+        if (nh == 0 || u < (unsigned)nh || flag[e] == 0) {
+            int seed = -1;
+            for (int r = 0; r < rounds && e + r < T; ++r) {
+                const int i = (int)(e + r) * kGroupQ + lane / kGroup;
+                int work = 0;
+                seed = search_group<PREC>(a.ix, a.src, a.prev, h, i, i < h.M, p2p, stk, seed, work);
+                if (a.hard && lane == 0) {
+                    const int cls = work > kHardWork ? 1 : (work > kHardWork / 2 ? 2 : 0);
+                    flag_out[e + r] = (unsigned char)cls;
+                    if (cls) {
+                        const int pos = atomicAdd(&a.st->hard_n[par ^ 1][cls - 1], 1);
+                        list_out[cls == 1 ? pos : T - 1 - pos] = (int)(e + r);
+                    }
+                }
+            }
         }
-        e = __shfl_sync(0xffffffffu, nx, 0);
+        u = __shfl_sync(0xffffffffu, nx, 0);
     }
 }
 
@@ -212,7 +242,8 @@ __global__ void __launch_bounds__(kCloseBlock) k_closest(Index ix, ClosestArgs a
         }
         // a non-finite x has no closest point: position 0, as a search that accepts nothing
         const bool finite = isfinite(xh[0] + xh[1] + xh[2]);
-        const int j = group_nn<PREC_FP64>(ix, xh, xl, bound, s_stk[threadIdx.x / kGroup], live && finite);
+        int work = 0;
+        const int j = group_nn<PREC_FP64>(ix, xh, xl, bound, s_stk[threadIdx.x / kGroup], live && finite, work);
         if (sorted != nullptr && finite) seed = j;
         if (live && (lane & (kGroup - 1)) == 0) {
             const float4 qq = __ldg(ix.pts + max(j, 0));

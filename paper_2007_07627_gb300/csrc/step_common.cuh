@@ -155,7 +155,7 @@ __device__ __forceinline__ void transform_query(const StepHead &h, float4 p, flo
 // the sums are bit-identical. Returns the correspondence.
 template <int PREC>
 __device__ __forceinline__ int search_group(const Index &ix, const float4 *src, int *prev, const StepHead &h, int i,
-                                            bool live, bool p2p, float2 *stk, int seed) {
+                                            bool live, bool p2p, float2 *stk, int seed, int &work) {
     float xh[3] = {0.0f, 0.0f, 0.0f}, xl[3] = {0.0f, 0.0f, 0.0f};
     float bound = __int_as_float(0x7f800000);
     int j0 = -1;
@@ -168,7 +168,7 @@ __device__ __forceinline__ int search_group(const Index &ix, const float4 *src, 
     }
     // (fricp_eval_pass_static also searches non-finite points, which it then rejects)
     const bool finite = isfinite(xh[0] + xh[1] + xh[2]);
-    int j = group_nn<PREC>(ix, xh, xl, bound, stk, live && finite);
+    int j = group_nn<PREC>(ix, xh, xl, bound, stk, live && finite, work);
     if (j < 0) j = j0 < 0 ? 0 : j0;   // nothing inside the cap
     if (live && (threadIdx.x & (kGroup - 1)) == 0) prev[i] = j;
     __syncwarp();
@@ -350,6 +350,15 @@ __device__ __forceinline__ bool accum_tile(const StepHead &h, PairState *st, con
     return last;
 }
 
+// The next pass's tile and search tickets start over; the lists of hard tickets
+// this pass used are empty again for the pass after the next (device_steps counts
+// this pass).
+__device__ __forceinline__ void reset_tickets(PairState *st) {
+    st->counter = 0u;
+    st->nn_next = 0u;
+    st->hard_n[(st->device_steps + 1) & 1][0] = st->hard_n[(st->device_steps + 1) & 1][1] = 0;
+}
+
 // Work of the block that completed a pass: the fixed-order reduction of the
 // tile records, then either the nu_max median (PH_INIT) or one solver step by
 // the block's first warp (team scratch: `team_sh`, kTeamScratch doubles of
@@ -364,8 +373,7 @@ __device__ __forceinline__ void finish_pass(const StepHead &h, PairState *st, co
         if (threadIdx.x == 0) {
             st->device_steps++;
             if (st->eval_counts) st->corr_passes++;
-            st->counter = 0u;   // the next pass's tile and search tickets start over
-            st->nn_next = 0u;
+            reset_tickets(st);
         }
     } else if (h.phase == PH_INIT) {
         const int n = h.M;
@@ -375,8 +383,7 @@ __device__ __forceinline__ void finish_pass(const StepHead &h, PairState *st, co
             st->device_steps++;
             if (st->eval_counts) st->corr_passes++;
             start_after_init(st, 0.5 * (lo + hi));
-            st->counter = 0u;   // the next pass's tile and search tickets start over
-            st->nn_next = 0u;
+            reset_tickets(st);
         }
     } else if (threadIdx.x < kTeamLanes) {
         solver_step(Team{team_sh}, st, sS, trace);   // resets the tickets in its copy of the state
