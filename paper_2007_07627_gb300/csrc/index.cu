@@ -750,7 +750,7 @@ __device__ __noinline__ bool tile_knn6(const Index &ix, int g, int i, bool live,
 struct NearK {
     float d;
     int j;
-    float bound;   // the K-th distance
+    float bound;   // upper bound of the K-th distance
     float spill;   // smallest distance that left the list
 };
 
@@ -785,7 +785,7 @@ __device__ __forceinline__ void near_scan(const Index &ix, const float xq[3], in
     }
     unsigned cm = __ballot_sync(FULL, d < INF);
     if (cm == 0u) return;
-    if (__popc(cm) <= 3) {   // a few: insert one by one
+    if (__popc(cm) <= 6) {   // a few: insert one by one
         while (cm) {
             const int src = __ffs(cm) - 1;
             cm &= cm - 1u;
@@ -818,79 +818,70 @@ __device__ __forceinline__ void near_scan(const Index &ix, const float xq[3], in
         for (int o = 16; o > 0; o >>= 1) out = fminf(out, __shfl_xor_sync(FULL, out, o));
         t.spill = fminf(t.spill, out);
     }
-    t.bound = __shfl_sync(FULL, t.d, K - 1);
+    t.bound = fminf(t.bound, __shfl_sync(FULL, t.d, K - 1));
 }
 
-// The K nearest of point i in lanes 0 .. K-1 (point `skip` left out). Returns 0 if they are the exact K,
-// 1 if float distances cannot tell, 2 if the stack would overflow.
-__device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3], int skip, int K, NearK &t, int *stk) {
+// The K nearest of point i in lanes 0 .. K-1 (point `skip` left out), all of them
+// within the squared distance `bound` (INF if none is known). Returns 0 if they
+// are the exact K, 1 if float distances cannot tell, 2 if the stack would overflow.
+//
+// The point's bucket and its sibling are scanned first; then the walk of group_nn
+// over the oriented boxes, by the whole warp: up to four nodes a round, eight
+// children each, and the buckets within the bound two at a time, nearest first.
+constexpr int kNearStack = kWarpStack;   // a round replaces up to 4 nodes by at most 32: below 9 levels x 32 + 8
+
+__device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3], int skip, int K, float bound,
+                                        NearK &t, int *stk) {
     const unsigned FULL = 0xffffffffu;
     const float INF = __int_as_float(0x7f800000);
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     const float zero[3] = {0.0f, 0.0f, 0.0f};
-    t.d = t.bound = t.spill = INF;
+    t.d = t.spill = INF;
+    t.bound = bound;
     t.j = -1;
-    const int depth = 31 - __clz(ix.L);
-    const int start = ix.L + i / kLeaf;
-    near_scan(ix, xq, skip, t, K, start, start ^ 1, depth > 0);   // the point's bucket and its sibling first
-    int sp;
-    {
-        int c = 0;
+    const int own = i / kLeaf;
+    near_scan(ix, xq, skip, t, K, ix.L + own, ix.L + (own ^ 1), ix.L > 1);
+    int sp = 0, base = 0;
+    bool live = lane >= 8 - ix.first && lane < 8;   // the first round: the nodes of the first level
+    for (;;) {
+        const bool leaf = base + 7 >= ix.leaf0;
+        const int pos = base + (lane & 7);
+        float key = INF;
         bool pass = false;
-        if (lane < depth - 1) {
-            c = (start >> (depth - 1 - lane)) ^ 1;
-            pass = box_d2(__ldg(ix.nodes + 2 * c), __ldg(ix.nodes + 2 * c + 1), xq, zero) * kShrink <= t.bound;
+        if (live && !(leaf && ((pos - ix.leaf0) ^ own) <= 1)) {   // the two buckets scanned first are done
+            key = obb_d2(obb_at(ix.obb, pos), xq, zero) * kObbShrink;
+            pass = key <= t.bound;
         }
-        const unsigned m = __ballot_sync(FULL, pass);
-        if (pass) stk[__popc(m & below)] = c;
-        sp = __popc(m);
-    }
-    __syncwarp();
-    while (sp > 0) {
-        const int k = min(32, sp);
-        const int node = (lane < k) ? stk[sp - 1 - lane] : 0;
+        const unsigned im = __ballot_sync(FULL, pass && !leaf);
+        if (sp + __popc(im) > kNearStack) return 2;
+        if (pass && !leaf) stk[sp + __popc(im & below)] = pos;
+        sp += __popc(im);
+        for (;;) {   // buckets, nearest first
+            unsigned m[2];
+#pragma unroll
+            for (int two = 0; two < 2; ++two) {
+                const bool in = pass && leaf && key <= t.bound;
+                m[two] = __reduce_min_sync(FULL, in ? (__float_as_uint(key) & ~31u) | lane : 0xffffffffu);
+                if (m[two] != 0xffffffffu && lane == (int)(m[two] & 31u)) pass = false;
+            }
+            if (m[0] == 0xffffffffu) break;
+            const bool two = m[1] != 0xffffffffu;
+            const int na = __shfl_sync(FULL, pos, m[0] & 31u), nb = __shfl_sync(FULL, pos, m[1] & 31u);
+            near_scan(ix, xq, skip, t, K, ix.L + na - ix.leaf0, ix.L + nb - ix.leaf0, two);
+        }
+        __syncwarp();
+        if (sp == 0) break;
+        const int k = min(4, sp), g = lane >> 3;
+        live = g < k;
+        base = live ? 8 * stk[sp - 1 - g] + 8 * ix.first - 56 : 0;
         sp -= k;
         __syncwarp();
-        // inner nodes at least two levels above the buckets expand to four grandchildren, others to two children
-        int c0 = 0, nc = 0;
-        bool leaf_ok = false;
-        if (node != 0) {
-            if (node < ix.L) {
-                const bool deep = 2 * node < ix.L;
-                c0 = deep ? 4 * node : 2 * node;
-                nc = deep ? 4 : 2;
-            } else {
-                leaf_ok = box_d2(__ldg(ix.nodes + 2 * node), __ldg(ix.nodes + 2 * node + 1), xq, zero) * kShrink
-                              <= t.bound &&
-                          obb_d2(obb_at(ix.obb, node - ix.L + ix.leaf0), xq, zero) * kObbShrink <= t.bound;
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            bool ok = false;
-            if (g < nc)
-                ok = box_d2(__ldg(ix.nodes + 2 * (c0 + g)), __ldg(ix.nodes + 2 * (c0 + g) + 1), xq, zero) * kShrink <=
-                     t.bound;
-            const unsigned mg = __ballot_sync(FULL, ok);
-            if (sp + __popc(mg) > kWarpStack) return 2;
-            if (ok) stk[sp + __popc(mg & below)] = c0 + g;
-            sp += __popc(mg);
-        }
-        unsigned lm = __ballot_sync(FULL, leaf_ok);
-        while (lm) {   // two buckets per pass: lanes 0-15 and 16-31
-            const int la = __ffs(lm) - 1;
-            lm &= lm - 1u;
-            const bool two = lm != 0u;
-            const int lb = two ? __ffs(lm) - 1 : la;
-            if (two) lm &= lm - 1u;
-            const int na = __shfl_sync(FULL, node, la), nb = __shfl_sync(FULL, node, lb);
-            near_scan(ix, xq, skip, t, K, na, nb, two);
-        }
-        __syncwarp();
     }
+    const float kth = __shfl_sync(FULL, t.d, K - 1);
     const float next = K < 32 ? __shfl_sync(FULL, t.d, K & 31) : t.spill;
-    return !(t.bound < INF) || (next <= t.bound * kTieWindow && next < INF) ? 1 : 0;   // not finite: distances beyond float
+    t.bound = kth;
+    return !(kth < INF) || (next <= kth * kTieWindow && next < INF) ? 1 : 0;
 }
 
 // The same selection by float distance: each lane keeps its seven nearest, sorted.
@@ -1043,7 +1034,7 @@ __global__ void __launch_bounds__(kKnnBlock) k_knn6_rest(Index ix, double *__res
         const float4 qi = __ldg(ix.pts + i);
         const float xq[3] = {qi.x, qi.y, qi.z};
         NearK t;
-        const int rc = near_knn(ix, i, xq, i, 6, t, s_stk[w]);
+        const int rc = near_knn(ix, i, xq, i, 6, __int_as_float(0x7f800000), t, s_stk[w]);
         __syncwarp();
         if (rc != 0) {
             Best6 b;
@@ -1094,15 +1085,15 @@ __global__ void __launch_bounds__(kKnnBlock) k_knn6_rest(Index ix, double *__res
 // original index); the normal is the eigenvector of the smallest eigenvalue of
 // the neighbourhood's covariance about its centroid, turned towards a viewpoint.
 //
-// k_normals: a warp takes up to 32 Morton-consecutive points.
-//   1. For each of them the whole warp finds the K nearest by float distance
-//      (near_knn: the traversal of warp_knn6, the sorted list one entry per
-//      lane, new buckets merged 32 candidates at a time). Float distances have a
+// k_normals: a block takes up to 32 Morton-consecutive points.
+//   1. Each warp finds the K nearest of its points by float distance, one point
+//      after the other (near_knn: the list sorted one entry per lane, buckets
+//      merged 32 candidates at a time). Float distances have a
 //      relative error below 4e-7, so the set is the exact one unless the
 //      (K+1)-th lies within 2e-6 of the K-th; those points (ties, and about one
 //      in 10^4 otherwise) are searched again with FP64 distances (warp_knn_k).
-//   2. Each lane takes one point: the covariance of its neighbours in FP64 and
-//      its smallest eigenvector (smallest_axis).
+//   2. Each lane of the first warp takes one point: the covariance of its
+//      neighbours in FP64 and its smallest eigenvector (smallest_axis).
 // GB300 issues an FP64 warp instruction once in 64 cycles however many lanes it
 // has, so FP64 work spread over a warp per point (distances, list comparisons,
 // covariance sums, 3.0 ms of k_knn_cov for 100,000 points) was the bound; with a
@@ -1344,21 +1335,37 @@ __device__ __forceinline__ void smallest_axis(const double e[6], double n[3]) {
     }
 }
 
-// Normals of `per_warp` (a power of two up to 32) Morton-consecutive points per
-// warp, turned so that n . (viewpoint - q) >= 0, written at the original index.
+// Normals of 4 x `per_warp` (up to 8) Morton-consecutive points per block, turned
+// so that n . (viewpoint - q) >= 0, written at the original index. Consecutive
+// points are close: the K nearest of one lie within its K-th distance plus the
+// step to the next, which bounds the next one's search from the start.
+constexpr int kNormalsPerWarp = 8;
+
 __global__ void __launch_bounds__(kKnnBlock) k_normals(Index ix, int K, int per_warp, double v0, double v1, double v2,
                                                        float *__restrict__ out, int *__restrict__ overflow) {
-    __shared__ int s_stk[kKnnBlock / 32][kWarpStack];
-    __shared__ int s_nbr[kKnnBlock / 32][32][33];
+    __shared__ int s_stk[kKnnBlock / 32][kWarpStack];   // kNearStack of it, but warp_knn_k takes all
+    __shared__ int s_nbr[32][33];
+    const float INF = __int_as_float(0x7f800000);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t i0 = ((int64_t)blockIdx.x * (kKnnBlock / 32) + w) * per_warp;
+    const int64_t b0 = (int64_t)blockIdx.x * (kKnnBlock / 32) * per_warp;
+    float bound = INF;
+    float last[3] = {0.0f, 0.0f, 0.0f};
     for (int p = 0; p < per_warp; ++p) {
-        const int64_t i = i0 + p;
+        const int64_t i = b0 + w * per_warp + p;
         if (i >= ix.n) break;   // uniform in the warp
         const float4 qi = __ldg(ix.pts + i);
         const float xq[3] = {qi.x, qi.y, qi.z};
+        if (bound < INF) {
+            const float dx = xq[0] - last[0], dy = xq[1] - last[1], dz = xq[2] - last[2];
+            const float r = sqrtf(bound) + sqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+            bound = r * r * (1.0f + 1e-5f);
+        }
         NearK t;
-        int rc = near_knn(ix, (int)i, xq, -1, K, t, s_stk[w]);
+        int rc = near_knn(ix, (int)i, xq, -1, K, bound, t, s_stk[w]);
+        bound = t.bound;
+        last[0] = xq[0];
+        last[1] = xq[1];
+        last[2] = xq[2];
         __syncwarp();
         if (rc == 1) {
             TopK e;
@@ -1366,17 +1373,18 @@ __global__ void __launch_bounds__(kKnnBlock) k_normals(Index ix, int K, int per_
             t.j = e.j;
         }
         if (rc == 2 && lane == 0) *overflow = 1;
-        s_nbr[w][p][lane] = rc == 2 ? (int)i : t.j;
+        s_nbr[w * per_warp + p][lane] = rc == 2 ? (int)i : t.j;
         __syncwarp();
     }
-    const int64_t i = i0 + lane;
-    if (lane >= per_warp || i >= ix.n) return;
+    __syncthreads();
+    const int64_t i = b0 + lane;
+    if (w != 0 || lane >= (kKnnBlock / 32) * per_warp || i >= ix.n) return;
     const float4 qi = __ldg(ix.pts + i);
     const double x = qi.x, y = qi.y, z = qi.z;
     // sums of the differences to the point and of their products
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, e[6] = {0, 0, 0, 0, 0, 0};
     for (int k = 0; k < K; ++k) {
-        const float4 q = __ldg(ix.pts + s_nbr[w][lane][k]);
+        const float4 q = __ldg(ix.pts + s_nbr[lane][k]);
         const double d0 = (double)q.x - x, d1 = (double)q.y - y, d2 = (double)q.z - z;
         s0 += d0;
         s1 += d1;
@@ -1788,9 +1796,9 @@ cudaError_t estimate_normals(const TargetDev *t, int k, const double viewpoint[3
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        // 32 points per warp use the FP64 units best; fewer while that leaves an SM less than 16 warps
-        int per_warp = 32;
-        while (per_warp > 4 && t->n / per_warp < (int64_t)16 * (sms > 0 ? sms : 152)) per_warp /= 2;
+        // 32 points per block fill the lanes of its FP64 part; fewer while that leaves an SM less than two blocks
+        int per_warp = kNormalsPerWarp;
+        while (per_warp > 1 && t->n < (int64_t)2 * (kKnnBlock / 32) * per_warp * (sms > 0 ? sms : 152)) per_warp /= 2;
         const int64_t per_block = (int64_t)per_warp * (kKnnBlock / 32);
         k_normals<<<(unsigned)((t->n + per_block - 1) / per_block), kKnnBlock, 0, s>>>(
             ix, K, per_warp, viewpoint[0], viewpoint[1], viewpoint[2], out_dev, flag);

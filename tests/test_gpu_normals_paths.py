@@ -70,9 +70,9 @@ def test_close_small_eigenvalues(fr, thin):
     _check(fr, Q, 16)
 
 
-@pytest.mark.parametrize("n", [3, 16, 33, 9728, 9729, 40000, 77825])
+@pytest.mark.parametrize("n", [3, 16, 33, 9728, 9729, 40000, 77825, 1217, 4864])
 def test_points_per_warp(fr, n):
-    """Sizes on both sides of the rule for 4, 8, 16 or 32 points per warp; few points, ragged ends."""
+    """Sizes on both sides of the rule for the points per block; few points, ragged ends."""
     g = np.random.default_rng(n)
     u = g.random((n, 2))
     Q = np.column_stack([u, 0.2 * np.sin(6 * u[:, 0]) * np.cos(5 * u[:, 1])]) + 3.0
