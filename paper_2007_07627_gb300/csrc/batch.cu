@@ -63,65 +63,71 @@ constexpr int kPlanThreads = 1024;
 constexpr int kOrderCounter = 0, kOrderStride = 1, kOrderTiles = 2;
 constexpr int kTileQ = 8;
 constexpr int kMaxSlots = 4096;
-constexpr int kSlotsPerThread = kMaxSlots / kPlanThreads;
+static_assert(kPlanThreads == 1024, "32 warps");
 
+// One thread per slot (a thread with four slots in turn paid four chains of
+// dependent loads, and the scan and the searches ran over all 4,096 offsets
+// whatever the number of slots: 20 us a step with 16 registrations).
 __global__ void __launch_bounds__(kPlanThreads) k_plan(const Slot *__restrict__ slots, int nslots,
                                                        StepHead *__restrict__ heads, int *__restrict__ done,
                                                        int *__restrict__ tile_slot, int *__restrict__ tile_local,
                                                        int max_tiles, BatchCtl *ctl) {
-    __shared__ int s_off[kMaxSlots + 1];
-    __shared__ int s_scan[kPlanThreads];
+    __shared__ int s_off[kMaxSlots];
+    __shared__ int s_warp[kPlanThreads / 32];
     __shared__ int s_active;
-    const int t = threadIdx.x;
+    const unsigned FULL = 0xffffffffu;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     if (t == 0) s_active = 0;
     __syncthreads();
-    // contiguous run of slots per thread: [t * kSlotsPerThread, ...)
-    int cnt[kSlotsPerThread];
-    int run = 0, act = 0;
-#pragma unroll
-    for (int k = 0; k < kSlotsPerThread; ++k) {
-        const int p = t * kSlotsPerThread + k;
-        cnt[k] = 0;
+    int carry = 0;
+    for (int b = 0; b < nslots; b += kPlanThreads) {
+        const int p = b + t;
+        int cnt = 0, d = 1, live = 0;
         if (p < nslots) {
-            const Slot sl = slots[p];
-            int d = 1;
-            if (sl.live) {
-                d = sl.st->done;
+            live = slots[p].live;
+            if (live) {
+                const PairState *st = slots[p].st;
+                d = st->done;
                 if (!d) {
-                    cnt[k] = sl.ntiles;
-                    load_head(sl.st, heads[p]);
-                    ++act;
+                    cnt = slots[p].ntiles;
+                    load_head(st, heads[p]);
                 }
             }
-            done[p] = sl.live && d;
+            done[p] = live && d;
         }
-        run += cnt[k];
-    }
-    if (act) atomicAdd(&s_active, act);
-    // inclusive scan of the per-thread runs (Hillis-Steele)
-    s_scan[t] = run;
-    __syncthreads();
-    for (int o = 1; o < kPlanThreads; o <<= 1) {
-        const int v = t >= o ? s_scan[t - o] : 0;
-        __syncthreads();
-        s_scan[t] += v;
-        __syncthreads();
-    }
-    int base = s_scan[t] - run;
+        const unsigned am = __ballot_sync(FULL, live && !d);
+        if (lane == 0 && am) atomicAdd(&s_active, __popc(am));
+        int incl = cnt;
 #pragma unroll
-    for (int k = 0; k < kSlotsPerThread; ++k) {
-        s_off[t * kSlotsPerThread + k] = base;
-        base += cnt[k];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += x;
+        }
+        if (lane == 31) s_warp[w] = incl;
+        __syncthreads();
+        int before = 0, total = 0;
+        {
+            int x = s_warp[lane];   // kPlanThreads / 32 = 32 warps
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, x, o);
+                if (lane >= o) x += y;
+            }
+            total = __shfl_sync(FULL, x, 31);
+            const int prev = __shfl_sync(FULL, x, w > 0 ? w - 1 : 0);
+            before = w > 0 ? prev : 0;
+        }
+        if (p < nslots) s_off[p] = carry + before + incl - cnt;
+        carry += total;
+        __syncthreads();
     }
-    if (t == kPlanThreads - 1) s_off[kMaxSlots] = s_scan[t];
-    __syncthreads();
-    int total = s_off[kMaxSlots];
+    int total = carry;
     if (total > max_tiles) {   // the host sizes the list for every live slot; keep the bound anyway
         if (t == 0) ctl->overflow = 1;
         total = 0;
     }
     for (int g = t; g < total; g += kPlanThreads) {
-        int lo = 0, hi = kMaxSlots;   // largest p with s_off[p] <= g (empty slots repeat offsets)
+        int lo = 0, hi = nslots;   // largest p with s_off[p] <= g (empty slots repeat offsets)
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (s_off[mid] <= g) lo = mid; else hi = mid;
