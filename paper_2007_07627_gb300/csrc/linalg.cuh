@@ -110,6 +110,16 @@ FRICP_HD inline double bitsd(unsigned long long b) {
 // x == +-0 by its bits (integer instructions, not the FP64 pipe)
 FRICP_HD inline bool is_zero_bits(double x) { return (dbits(x) << 1) == 0ull; }
 
+// Comparisons on the bits: non-negative doubles order as integers, and an FP64
+// comparison occupies the FP64 pipe (64 cycles) like any other instruction.
+FRICP_HD inline long long sbits(double x) { return (long long)dbits(x); }
+FRICP_HD inline bool is_positive(double x) { return sbits(x) > 0 && dbits(x) <= 0x7ff0000000000000ull; }   // x > 0
+FRICP_HD inline bool is_finite(double x) { return (dbits(x) & 0x7fffffffffffffffull) < 0x7ff0000000000000ull; }
+// lo < x < hi for constants 0 < lo < hi (false for NaN)
+FRICP_HD inline bool within(double x, double lo, double hi) { return sbits(x) > sbits(lo) && sbits(x) < sbits(hi); }
+// x < c for x >= 0 or NaN and a constant c > 0
+FRICP_HD inline bool below(double x, double c) { return dbits(x) < dbits(c); }
+
 FRICP_HD inline void hat3(const double a[3], double H[9]) {
     H[0] = 0.0;   H[1] = -a[2]; H[2] = a[1];
     H[3] = a[2];  H[4] = 0.0;   H[5] = -a[0];
@@ -144,8 +154,7 @@ FRICP_HD inline void t_mul33(const Team &tm, const double *A, const double *B, d
 // outside the float range fall back to the IEEE operations. The steps are
 // written with explicit fma, so the host build rounds exactly as the device.
 FRICP_HD inline double rcp64(double a) {
-    const double fa = fabs(a);
-    if (!(fa > 1e-30 && fa < 1e30)) return 1.0 / a;
+    if (!within(fabs(a), 1e-30, 1e30)) return 1.0 / a;
     double y = (double)(1.0f / (float)a);
     y = fma(y, fma(-a, y, 1.0), y);
     y = fma(y, fma(-a, y, 1.0), y);
@@ -153,7 +162,7 @@ FRICP_HD inline double rcp64(double a) {
 }
 
 FRICP_HD inline double rsqrt64(double a) {
-    if (!(a > 1e-30 && a < 1e30)) return 1.0 / sqrt(a);
+    if (!within(a, 1e-30, 1e30)) return 1.0 / sqrt(a);
     double y = (double)(1.0f / sqrtf((float)a));
     y = y * fma(-0.5, (a * y) * y, 1.5);
     y = y * fma(-0.5, (a * y) * y, 1.5);
@@ -164,7 +173,7 @@ FRICP_HD inline double rsqrt64(double a) {
 // a = sin th / th, b = (1 - cos th) / th^2, c = (th - sin th) / th^3,
 // by their Taylor series below th = 1e-2 (truncation < 1e-21).
 FRICP_HD inline void exp_coeffs(double th2, double *a, double *b, double *c) {
-    if (th2 < 1e-4) {
+    if (below(th2, 1e-4)) {   // th2 >= 0
         *a = 1.0 - th2 * (1.0 / 6.0) * (1.0 - th2 * (1.0 / 20.0) * (1.0 - th2 * (1.0 / 42.0)));
         *b = 0.5 * (1.0 - th2 * (1.0 / 12.0) * (1.0 - th2 * (1.0 / 30.0) * (1.0 - th2 * (1.0 / 56.0))));
         *c = (1.0 / 6.0) * (1.0 - th2 * (1.0 / 20.0) * (1.0 - th2 * (1.0 / 42.0) * (1.0 - th2 * (1.0 / 72.0))));
@@ -217,13 +226,13 @@ FRICP_HD inline void se3_log(const Team &tm, const double *T, double xi[6], doub
     t_load(T, R);
     const double v0 = 0.5 * (R[7] - R[5]), v1 = 0.5 * (R[2] - R[6]), v2 = 0.5 * (R[3] - R[1]);
     const double sn2 = fma(v2, v2, fma(v1, v1, v0 * v0));
-    const double isn = sn2 > 0.0 ? rsqrt64(sn2) : 0.0;   // 1 / sin th (unused when sin th = 0)
+    const double isn = is_positive(sn2) ? rsqrt64(sn2) : 0.0;   // 1 / sin th (unused when sin th = 0)
     const double sn = sn2 * isn;
     const double cs = 0.5 * (R[0] + R[4] + R[8] - 1.0);
     const double th = atan2(sn, cs);
     const double th2 = th * th;
     double wv[3];
-    if (th < 1e-2) {
+    if (below(th, 1e-2)) {   // th in [0, pi]
         // th / sin th = 1 + th^2/6 + 7 th^4/360 + 31 th^6/15120
         const double f = 1.0 + th2 * (1.0 / 6.0) + th2 * th2 * (7.0 / 360.0) + th2 * th2 * th2 * (31.0 / 15120.0);
         wv[0] = f * v0; wv[1] = f * v1; wv[2] = f * v2;
@@ -253,7 +262,7 @@ FRICP_HD inline void se3_log(const Team &tm, const double *T, double xi[6], doub
         wv[0] = f * v0; wv[1] = f * v1; wv[2] = f * v2;
     }
     double e;
-    if (th < 1e-2) {
+    if (below(th, 1e-2)) {
         e = 1.0 / 12.0 + th2 * (1.0 / 720.0) + th2 * th2 * (1.0 / 30240.0);
     } else {
         // sin th and cos th are sn and cs themselves (R orthogonal): no sincos
@@ -412,23 +421,48 @@ FRICP_HD inline bool procrustes_rotation(const Team &tm, const double *H, double
     // Newton on SO(3): R <- exp(w^) R with (tr(A) I - sym(A)) w = vee(A - A^T), A = R H
     for (int it = 0; it < 2; ++it) {
         t_mul33(tm, R, H, Am);
-        double a[9];
-        t_load(Am, a);
-        const double g[3] = {a[5] - a[7], a[6] - a[2], a[1] - a[3]};
-        const double tr = a[0] + a[4] + a[8];
-        const double k00 = tr - a[0], k11 = tr - a[4], k22 = tr - a[8];
-        const double k01 = -0.5 * (a[1] + a[3]), k02 = -0.5 * (a[2] + a[6]), k12 = -0.5 * (a[5] + a[7]);
-        const double c00 = fma(k11, k22, -(k12 * k12)), c01 = fma(k02, k12, -(k01 * k22));
-        const double c02 = fma(k01, k12, -(k02 * k11)), c11 = fma(k00, k22, -(k02 * k02));
-        const double c12 = fma(k01, k02, -(k00 * k12)), c22 = fma(k00, k11, -(k01 * k01));
-        const double det = fma(k02, c02, fma(k01, c01, k00 * c00));
-        if (!(det > 0.0) || !(k00 > 0.0) || !isfinite(det)) return false;
+        // the scalars of the 3x3 system one per lane: g (3), the off-diagonal of K (01, 02, 12) and its diagonal ...
+        const double tr = Am[0] + Am[4] + Am[8];
+        for (int e = tm.lane(); e < 9; e += tm.size()) {
+            const int ix = e < 3 ? (e == 0 ? 5 : (e == 1 ? 6 : 1)) : (e < 6 ? (e == 3 ? 1 : (e == 4 ? 2 : 5)) : 0);
+            const int iy = e < 3 ? (e == 0 ? 7 : (e == 1 ? 2 : 3)) : (e < 6 ? (e == 3 ? 3 : (e == 4 ? 6 : 7)) : 4 * (e - 6));
+            const double x = e < 6 ? Am[ix] : tr, y = (e < 3 || e >= 6) ? -Am[iy] : Am[iy];
+            N[e] = (x + y) * ((e >= 3 && e < 6) ? -0.5 : 1.0);
+        }
+        tm.sync();
+        // ... its cofactors (00, 01, 02, 11, 12, 22) ...
+        for (int e = tm.lane(); e < 6; e += tm.size()) {
+            const int pi = e == 0 ? 7 : (e == 1 ? 4 : (e == 2 || e == 4 ? 3 : 6));
+            const int qi = e == 0 || e == 3 ? 8 : (e == 4 ? 4 : (e == 5 ? 7 : 5));
+            const int ri = e == 0 ? 5 : (e == 1 || e == 5 ? 3 : (e == 4 ? 6 : 4));
+            const int si = e == 0 || e == 4 ? 5 : (e == 1 ? 8 : (e == 2 ? 7 : (e == 3 ? 4 : 3)));
+            Tm[e] = fma(N[pi], N[qi], -(N[ri] * N[si]));
+        }
+        tm.sync();
+        const double det = fma(N[4], Tm[2], fma(N[3], Tm[1], N[6] * Tm[0]));
+        if (!is_positive(det) || !is_positive(N[6]) || !is_finite(det)) return false;
         const double idet = rcp64(det);
-        const double wv[3] = {fma(c02, g[2], fma(c01, g[1], c00 * g[0])) * idet,
-                              fma(c12, g[2], fma(c11, g[1], c01 * g[0])) * idet,
-                              fma(c22, g[2], fma(c12, g[1], c02 * g[0])) * idet};
+        // ... and w = K^-1 g
+        for (int e = tm.lane(); e < 3; e += tm.size()) {
+            const double c0 = Tm[e], c1 = Tm[e == 0 ? 1 : 2 + e], c2 = Tm[e == 0 ? 2 : 3 + e];
+            E[e] = fma(c2, N[2], fma(c1, N[1], c0 * N[0])) * idet;
+        }
+        tm.sync();
+        const double wv[3] = {E[0], E[1], E[2]};
+        const double th2 = fma(wv[2], wv[2], fma(wv[1], wv[1], wv[0] * wv[0]));
         double ea, eb, ec;
-        exp_coeffs(fma(wv[2], wv[2], fma(wv[1], wv[1], wv[0] * wv[0])), &ea, &eb, &ec);
+        if (below(th2, 1e-4)) {   // the series of exp_coeffs, one per lane
+            for (int e = tm.lane(); e < 2; e += tm.size()) {
+                const double k1 = e == 0 ? 1.0 / 6.0 : 1.0 / 12.0, k2 = e == 0 ? 1.0 / 20.0 : 1.0 / 30.0;
+                const double k3 = e == 0 ? 1.0 / 42.0 : 1.0 / 56.0;
+                E[3 + e] = (e == 0 ? 1.0 : 0.5) * (1.0 - th2 * k1 * (1.0 - th2 * k2 * (1.0 - th2 * k3)));
+            }
+            tm.sync();
+            ea = E[3];
+            eb = E[4];
+        } else {
+            exp_coeffs(th2, &ea, &eb, &ec);
+        }
         double Wr[9];
         hat3(wv, Wr);
         t_store<9>(tm, W, Wr);
@@ -465,10 +499,10 @@ FRICP_HD inline bool anderson_lstsq(const Team &tm, double *Dm, int mk, double t
 #pragma unroll
         for (int i = 0; i < 6; ++i) v[i] = (i < j) ? 0.0 : Dm[6 * j + i];
         const double nrm2 = dot6(v, v);
-        const double nrm = nrm2 > 0.0 ? nrm2 * rsqrt64(nrm2) : 0.0;
+        const double nrm = is_positive(nrm2) ? nrm2 * rsqrt64(nrm2) : 0.0;
         const double alpha = -copysign(nrm, v[j]);
         Rd[j] = alpha;
-        if (nrm == 0.0) continue;
+        if (is_zero_bits(nrm)) continue;
         // v = x - alpha e_j has |v_j| = |x_j| + nrm, so v.v = 2 (nrm^2 + |x_j| nrm)
         const double vv2 = fma(fabs(v[j]), nrm, nrm2);
         v[j] -= alpha;
@@ -486,14 +520,16 @@ FRICP_HD inline bool anderson_lstsq(const Team &tm, double *Dm, int mk, double t
         }
         tm.sync();
     }
-    double rmax = 0.0, rmin = INFINITY;
+    // min and max of |R_jj| on the bits (a NaN orders above infinity: not finite, as its theta would be)
+    unsigned long long bmax = 0ull, bmin = 0x7ff0000000000000ull;
 #pragma unroll
     for (int j = 0; j < kMaxM; ++j) {
         if (j >= mk) continue;
-        rmax = fmax(rmax, fabs(Rd[j]));
-        rmin = fmin(rmin, fabs(Rd[j]));
+        const unsigned long long b = dbits(Rd[j]) & 0x7fffffffffffffffull;
+        bmax = b > bmax ? b : bmax;
+        bmin = b < bmin ? b : bmin;
     }
-    if (!isfinite(rmax) || rmax == 0.0 || rmin < 1e-14 * rmax) return false;
+    if (bmax >= 0x7ff0000000000000ull || bmax == 0ull || bmin < dbits(1e-14 * bitsd(bmax))) return false;
     // 1 / R_jj, one per lane
     for (int j = tm.lane(); j < mk; j += tm.size()) {
         double rj = Rd[0];
@@ -512,7 +548,7 @@ FRICP_HD inline bool anderson_lstsq(const Team &tm, double *Dm, int mk, double t
         for (int c = j + 1; c < kMaxM; ++c)
             if (c < mk) acc = fma(-Dm[6 * c + j], theta[c], acc);
         theta[j] = acc * w[j];
-        if (!isfinite(theta[j])) return false;
+        if (!is_finite(theta[j])) return false;
     }
     return true;
 }
@@ -559,7 +595,7 @@ FRICP_HD inline bool chol6_solve(const Team &tm, const double *A, const double *
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
         const double d = L[7 * j];
-        if (!(d > 0.0) || !isfinite(d)) return false;
+        if (!is_positive(d) || !is_finite(d)) return false;
         il[j] = rsqrt64(d);   // 1 / L_jj
         tm.sync();
         for (int i = j + 1 + tm.lane(); i < 6; i += tm.size()) L[6 * i + j] *= il[j];
@@ -611,10 +647,10 @@ FRICP_HD inline bool chol6_solve(const Team &tm, const double *A, const double *
 FRICP_HD inline void p2pl_chain(const Team &tm, const double xi[6], double *K, double *w) {
     const double *d = xi, *u = xi + 3;
     const double th2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]));
-    if (th2 == 0.0 || th2 < 1e-12) {   // the rare near-identity cases, by every lane alike
+    if (below(th2, 1e-12)) {   // the rare near-identity cases, by every lane alike (th2 >= 0)
         double Kr[36];
         for (int i = 0; i < 36; ++i) Kr[i] = 0.0;
-        if (th2 == 0.0) {
+        if (is_zero_bits(th2)) {
             for (int j = 0; j < 3; ++j) {
                 Kr[6 * j + j] = 1.0;
                 Kr[6 * (3 + j) + 3 + j] = 1.0;

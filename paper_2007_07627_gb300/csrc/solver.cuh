@@ -152,15 +152,12 @@ __device__ inline void anderson_step(const Team &tm, const PairState *st, int mk
     if (mk <= 0) return;
     double *Dm = tm.sh + kShD, *xo = tm.sh + kShX;
     tm.sync();
-    // column c of D (c < mk): F^(k-c) - F^(k-c-1); column kMaxM: f = F^(k)
-    for (int c = tm.lane(); c <= kMaxM; c += tm.size()) {
-        if (c == kMaxM) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) Dm[6 * c + i] = ((i < 3) ? wrot : 1.0) * st->Fh[nw][i];
-        } else if (c < mk) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i)
-                Dm[6 * c + i] = ((i < 3) ? wrot : 1.0) * (st->Fh[nw - c][i] - st->Fh[nw - c - 1][i]);
+    // column c of D (c < mk): F^(k-c) - F^(k-c-1); column kMaxM: f = F^(k); one entry per lane
+    for (int e = tm.lane(); e < 6 * (kMaxM + 1); e += tm.size()) {
+        const int c = e / 6, i = e - 6 * c;
+        if (c < mk || c == kMaxM) {
+            const double f = st->Fh[c == kMaxM ? nw : nw - c][i];
+            Dm[e] = (i < 3 ? wrot : 1.0) * (c == kMaxM ? f : f - st->Fh[nw - c - 1][i]);
         }
     }
     tm.sync();
@@ -188,7 +185,7 @@ __device__ inline void anderson_step(const Team &tm, const PairState *st, int mk
 // T (12) written to scratch. w: 80 doubles of scratch.
 __device__ inline bool align_from_sums(const Team &tm, const PairState *st, const double *S, double *T, double *w) {
     const double W = S[0];
-    if (!(W > 0.0) || !isfinite(W)) return false;
+    if (!is_positive(W) || !is_finite(W)) return false;
     double *pq = w, *H = w + 8, *pw = w + 18;   // pq: pbar (3), qbar (3)
     tm.sync();
     for (int e = tm.lane(); e < 6; e += tm.size()) pq[e] = S[1 + e] / W;
@@ -226,8 +223,10 @@ __device__ inline void p2p_continue(const Team &tm, PairState *st, double E, con
         return;
     }
     copy_n(st->Tp, T, 12);
-    double fro = 0.0;
-    for (int i = 0; i < 12; ++i) fro = fma(st->Tk[i] - T[i], st->Tk[i] - T[i], fro);
+    double fro = 0.0, *dT = tm.sh + kShX;
+    for (int i = tm.lane(); i < 12; i += tm.size()) dT[i] = st->Tk[i] - T[i];
+    tm.sync();
+    for (int i = 0; i < 12; ++i) fro = fma(dT[i], dT[i], fro);
     if (fro < st->eps * st->eps) {
         p2p_stage_end(tm, st, 0);
         return;
