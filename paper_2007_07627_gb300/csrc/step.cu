@@ -18,7 +18,7 @@ namespace fricp {
 namespace {
 
 constexpr int kHardWork = 64;    // rounds and scans (24 on average) above which a ticket is hard, half of it: fairly hard
-constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket of a first pass
+constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket of a first pass (see k_nn)
 
 // Search kernel: persistent warps take runs of Morton-adjacent queries, four
 // queries at a time (search_group). Writes prev[i] = this pass's correspondence
@@ -27,8 +27,10 @@ constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket
 // queries in flight stay in one window of the Morton order; each query's result
 // depends only on the query. A warm pass takes four queries per ticket (runs of
 // sixteen left the last tickets running alone: 335 us against 218 us, ellipsoids,
-// M = 200,000); a first pass takes longer runs, whose queries start from the
-// result of the one before.
+// M = 200,000). The first pass of a large source takes longer runs, whose queries
+// start from the result of the one before, once there are 16 tickets per warp
+// (eval_pass, M = 200,000: 623 us with single tickets, 635 with runs of two, 695
+// with four; fricp_closest_points, M = 1M: 2.27, 1.81, 1.69 ms).
 //
 // A few queries (outliers about equally far from a large part of the target) walk
 // ten times the average, and one that starts late runs on alone. They are the same
@@ -36,8 +38,11 @@ constexpr int kColdRounds = 4;   // runs of up to 4 x kGroupQ queries per ticket
 // takes them first. Every ticket is searched once either way. (Ellipsoids, M =
 // 200,000: 197 -> 157 us; field, M = 80,000: 91 -> 82 us; thresholds of 48, 96 and
 // 160: 158, 161, 169 us.)
+//
+// Four blocks per SM in FP64 mode (five spill: 156 -> 167 us), five in the others
+// (field, M = 80,000, FP32: 80 -> 75-78 us).
 template <int PREC>
-__global__ void __launch_bounds__(kBlock) k_nn(StepArgs a) {
+__global__ void __launch_bounds__(kBlock, PREC == PREC_FP64 ? 4 : 5) k_nn(StepArgs a) {
     __shared__ StepHead h;
     __shared__ float2 s_stk[kBlock / kGroup][kGroupStack];
     if (threadIdx.x == 0) load_head(a.st, h);
@@ -48,7 +53,7 @@ __global__ void __launch_bounds__(kBlock) k_nn(StepArgs a) {
     float2 *stk = s_stk[threadIdx.x / kGroup];
     const unsigned warps = gridDim.x * (kBlock / 32);
     const int step = a.st->device_steps;
-    const int rounds = step == 0 ? max(1, min(kColdRounds, (int)(h.M / (2 * kGroupQ * warps)))) : 1;
+    const int rounds = step == 0 ? max(1, min(kColdRounds, (int)(h.M / (16 * kGroupQ * warps)))) : 1;
     // hard tickets listed by the pass before: class 0 from the front of its list, class 1 from the back
     const int T = (int)search_tickets(h.M), par = step & 1;
     const int n0 = a.hard ? a.st->hard_n[par][0] : 0, n1 = a.hard ? a.st->hard_n[par][1] : 0, nh = n0 + n1;
