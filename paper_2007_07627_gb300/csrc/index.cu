@@ -87,7 +87,7 @@ __global__ void k_box_partial(const float *__restrict__ x, const float *__restri
 
 // One block folds the per-block records: thread t takes records t, t+256, ...,
 // then a fixed shared-memory tree (deterministic order).
-__global__ void k_box_final(const BoxPartial *parts, int nparts, BoxPartial *out) {
+__global__ void k_box_final(const BoxPartial *parts, int nparts, BoxPartial *out, BoxPartial *host_out) {
     __shared__ float slo[3][kRedBlock], shi[3][kRedBlock];
     __shared__ double ssum[3][kRedBlock];
     __shared__ int sbad[kRedBlock];
@@ -129,6 +129,7 @@ __global__ void k_box_final(const BoxPartial *parts, int nparts, BoxPartial *out
         }
         r.bad = sbad[0];
         *out = r;
+        *host_out = r;   // pinned host memory: no copy of its own in the stream
     }
 }
 
@@ -140,12 +141,16 @@ __device__ __forceinline__ unsigned expand_bits10(unsigned v) {
     return v;
 }
 
-__global__ void k_morton(const float *__restrict__ x, int64_t n, float3 lo, float3 inv_ext,
+// Keys from the box k_box_final wrote: the host need not wait for it.
+__global__ void k_morton(const float *__restrict__ x, int64_t n, const BoxPartial *__restrict__ box,
                          unsigned *__restrict__ code, int *__restrict__ idx) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float c[3] = {(x[3 * i] - lo.x) * inv_ext.x, (x[3 * i + 1] - lo.y) * inv_ext.y,
-                        (x[3 * i + 2] - lo.z) * inv_ext.z};
+    float c[3];
+    for (int a = 0; a < 3; ++a) {
+        const float ext = box->hi[a] - box->lo[a];
+        c[a] = (x[3 * i + a] - box->lo[a]) * (ext > 0.0f ? 1.0f / ext : 0.0f);
+    }
     unsigned k[3];
     for (int a = 0; a < 3; ++a) k[a] = (unsigned)fminf(fmaxf(c[a] * 1024.0f, 0.0f), 1023.0f);
     code[i] = (expand_bits10(k[0]) << 2) | (expand_bits10(k[1]) << 1) | expand_bits10(k[2]);
@@ -1517,35 +1522,51 @@ __global__ void __launch_bounds__(256) k_median_pass(const double *v0, const dou
     }
 }
 
-struct BoxResult {
-    float lo[3], hi[3];
-    double sum[3];
-    int bad;
+// Bounding box, sum and validity of n points, on the device (parts: freed by the
+// caller on s) and in pinned host memory of this thread, which wait_box waits for:
+// what is queued in between runs meanwhile. Every start_box that succeeded is
+// followed by a wait_box before the next.
+struct BoxStage {
+    BoxPartial *h = nullptr;
+    cudaEvent_t ev = nullptr;
 };
 
-cudaError_t reduce_box(const float *x, const float *nrm, int64_t n, cudaStream_t s, BoxResult *res,
-                       int zero_normals_ok = 0) {
+BoxStage &box_stage() {
+    thread_local BoxStage b;
+    if (b.h == nullptr && cudaMallocHost(&b.h, sizeof(BoxPartial)) != cudaSuccess) b.h = nullptr;
+    if (b.ev == nullptr && cudaEventCreateWithFlags(&b.ev, cudaEventDisableTiming) != cudaSuccess) b.ev = nullptr;
+    return b;
+}
+
+cudaError_t start_box(const float *x, const float *nrm, int64_t n, cudaStream_t s, BoxPartial **parts_out,
+                      const BoxPartial **box_out, int zero_normals_ok = 0) {
+    BoxStage &st = box_stage();
+    if (st.h == nullptr || st.ev == nullptr) return cudaErrorMemoryAllocation;
     int nb = (int)std::min<int64_t>((n + kRedBlock - 1) / kRedBlock, 1024);
     if (nb < 1) nb = 1;
     BoxPartial *parts = nullptr;
     cudaError_t e = pool_alloc(&parts, sizeof(BoxPartial) * (nb + 1), s);
     if (e != cudaSuccess) return e;
     k_box_partial<<<nb, kRedBlock, 0, s>>>(x, nrm, n, parts, zero_normals_ok);
-    k_box_final<<<1, kRedBlock, 0, s>>>(parts, nb, parts + nb);
+    k_box_final<<<1, kRedBlock, 0, s>>>(parts, nb, parts + nb, st.h);
     counters().launches += 2;
-    BoxPartial h;
-    e = cudaMemcpyAsync(&h, parts + nb, sizeof(BoxPartial), cudaMemcpyDeviceToHost, s);
+    e = cudaGetLastError();
     counters().d2h += sizeof(BoxPartial);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(parts, s);
-    if (e != cudaSuccess) return e;
-    for (int a = 0; a < 3; ++a) {
-        res->lo[a] = h.lo[a];
-        res->hi[a] = h.hi[a];
-        res->sum[a] = h.sum[a];
+    if (e == cudaSuccess) e = cudaEventRecord(st.ev, s);
+    if (e != cudaSuccess) {
+        cudaFreeAsync(parts, s);
+        return e;
     }
-    res->bad = h.bad;
-    return cudaGetLastError();
+    *parts_out = parts;
+    *box_out = parts + nb;
+    return cudaSuccess;
+}
+
+cudaError_t wait_box(BoxPartial *res) {
+    BoxStage &st = box_stage();
+    const cudaError_t e = cudaEventSynchronize(st.ev);
+    if (e == cudaSuccess) *res = *st.h;
+    return e;
 }
 
 // Kernels one sort of n keys launches, for the launch counter: read off a capture
@@ -1579,7 +1600,7 @@ int64_t sort_launches(void *tmp, size_t tb, unsigned *code, unsigned *code2, int
 }
 
 // Morton order of n points: returns the permutation (device, caller frees).
-cudaError_t morton_order(const float *x, int64_t n, const BoxResult &bx, cudaStream_t s, int **order_out) {
+cudaError_t morton_order(const float *x, int64_t n, const BoxPartial *box, cudaStream_t s, int **order_out) {
     unsigned *code = nullptr, *code2 = nullptr;
     int *idx = nullptr, *idx2 = nullptr;
     void *tmp = nullptr;
@@ -1589,12 +1610,7 @@ cudaError_t morton_order(const float *x, int64_t n, const BoxResult &bx, cudaStr
     if (e == cudaSuccess) e = pool_alloc(&idx, 4 * n, s);
     if (e == cudaSuccess) e = pool_alloc(&idx2, 4 * n, s);
     if (e == cudaSuccess) {
-        float3 lo = make_float3(bx.lo[0], bx.lo[1], bx.lo[2]);
-        float ext[3];
-        for (int a = 0; a < 3; ++a) ext[a] = bx.hi[a] - bx.lo[a];
-        float3 inv = make_float3(ext[0] > 0 ? 1.0f / ext[0] : 0.0f, ext[1] > 0 ? 1.0f / ext[1] : 0.0f,
-                                 ext[2] > 0 ? 1.0f / ext[2] : 0.0f);
-        k_morton<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, lo, inv, code, idx);
+        k_morton<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, box, code, idx);
         counters().launches += 1;
         e = cub::DeviceRadixSort::SortPairs(nullptr, tb, code, code2, idx, idx2, (int)n, 0, 30, s);
     }
@@ -1619,18 +1635,12 @@ cudaError_t morton_order(const float *x, int64_t n, const BoxResult &bx, cudaStr
 
 cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cudaStream_t s, TargetDev *t,
                          int *bad_input) {
-    BoxResult bx;
-    cudaError_t e = reduce_box(q_dev, n_dev, n, s, &bx);
+    BoxPartial *parts = nullptr;
+    const BoxPartial *box = nullptr;
+    cudaError_t e = start_box(q_dev, n_dev, n, s, &parts, &box);
     if (e != cudaSuccess) return e;
-    *bad_input = bx.bad;
-    if (bx.bad) return cudaSuccess;
     t->n = n;
     t->has_normals = n_dev != nullptr;
-    for (int a = 0; a < 3; ++a) {
-        t->lo[a] = bx.lo[a];
-        t->hi[a] = bx.hi[a];
-        t->centroid[a] = bx.sum[a] / (double)n;
-    }
     const int64_t buckets = (n + kLeaf - 1) / kLeaf;
     int L = 1;
     while (L < buckets) L *= 2;
@@ -1638,8 +1648,22 @@ cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cuda
     t->E_Q = -1.0;
     t->H_Q = -1.0;
     int *order = nullptr;
-    e = morton_order(q_dev, n, bx, s, &order);
-    if (e != cudaSuccess) return e;
+    e = morton_order(q_dev, n, box, s, &order);
+    cudaFreeAsync(parts, s);
+    BoxPartial bx;
+    const cudaError_t eb = wait_box(&bx);
+    if (e == cudaSuccess) e = eb;
+    if (e != cudaSuccess || bx.bad) {   // bad coordinates: their keys and order are of no use
+        if (order) cudaFreeAsync(order, s);
+        *bad_input = e == cudaSuccess;
+        return e;
+    }
+    *bad_input = 0;
+    for (int a = 0; a < 3; ++a) {
+        t->lo[a] = bx.lo[a];
+        t->hi[a] = bx.hi[a];
+        t->centroid[a] = bx.sum[a] / (double)n;
+    }
     e = pool_alloc(&t->pts, sizeof(float4) * n, s);
     if (e == cudaSuccess && n_dev) e = pool_alloc(&t->nrm, sizeof(float4) * n, s);
     if (e == cudaSuccess) e = pool_alloc(&t->nodes, sizeof(float4) * 4 * ((size_t)L + ((wide_leaf(L) + L + 7) / 8) * 8), s);
@@ -1816,23 +1840,31 @@ cudaError_t estimate_normals(const TargetDev *t, int k, const double viewpoint[3
 
 cudaError_t prepare_source(const float *p_dev, int64_t m, cudaStream_t s, float4 *src_out, float lo[3],
                            float hi[3], int *bad_input, const float *n_dev, float4 *nrm_out) {
-    BoxResult bx;
-    cudaError_t e = reduce_box(p_dev, n_dev, m, s, &bx, 1);   // a zero source normal: no normal at that point
+    BoxPartial *parts = nullptr;
+    const BoxPartial *box = nullptr;
+    cudaError_t e = start_box(p_dev, n_dev, m, s, &parts, &box, 1);   // a zero source normal: no normal at that point
     if (e != cudaSuccess) return e;
-    *bad_input = bx.bad;
-    if (bx.bad) return cudaSuccess;
-    for (int a = 0; a < 3; ++a) {
-        lo[a] = bx.lo[a];
-        hi[a] = bx.hi[a];
-    }
     int *order = nullptr;
-    e = morton_order(p_dev, m, bx, s, &order);
-    if (e != cudaSuccess) return e;
+    e = morton_order(p_dev, m, box, s, &order);
+    cudaFreeAsync(parts, s);
+    BoxPartial bx;
+    if (e != cudaSuccess) {
+        wait_box(&bx);
+        return e;
+    }
     k_gather<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(p_dev, n_dev, order, m, src_out, nrm_out);
     counters().launches += 1;
     e = cudaGetLastError();
     cudaFreeAsync(order, s);
-    return e;
+    const cudaError_t eb = wait_box(&bx);
+    if (e == cudaSuccess) e = eb;
+    if (e != cudaSuccess) return e;
+    *bad_input = bx.bad;
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = bx.lo[a];
+        hi[a] = bx.hi[a];
+    }
+    return cudaSuccess;
 }
 
 }  // namespace fricp
