@@ -64,18 +64,6 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
     }
     fricp_status rs = FRICP_OK;
     cudaError_t e = cudaSuccess;
-    if (use_graph) {
-        const int64_t before = counters().launches;   // capture records launches, it does not run them
-        e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            for (int k = 0; k < chunk; ++k) fricp::launch_step(a, variant, prec, ntiles, s);
-            e = cudaStreamEndCapture(s, &graph.g);
-        }
-        counters().launches = before;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&graph.exec, graph.g, 0);
-        if (e != cudaSuccess) rs = cuda_fail(e, "capturing the step graph");
-    }
-    const int64_t per_replay = use_graph && graph.g ? graph_kernel_nodes(graph.g) : 0;
     int64_t steps = 0;
     *pass_ms = 0.0;
     *search_ms = 0.0;
@@ -107,6 +95,25 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
                 for (auto &ev : iev) cudaEventDestroy(ev);
         }
     }
+    // The GPU runs the first steps while the host captures the graph of the others
+    // (a step past the end does nothing; small step budgets are kept to the step).
+    if (rs == FRICP_OK && use_graph && init_m == 0 && prm.max_steps >= 4096) {
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = fricp::launch_step(a, variant, prec, ntiles, s);
+        if (e != cudaSuccess) rs = cuda_fail(e, "launching step");
+        steps = 2;
+    }
+    if (rs == FRICP_OK && use_graph) {
+        const int64_t before = counters().launches;   // capture records launches, it does not run them
+        e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            for (int k = 0; k < chunk; ++k) fricp::launch_step(a, variant, prec, ntiles, s);
+            e = cudaStreamEndCapture(s, &graph.g);
+        }
+        counters().launches = before;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&graph.exec, graph.g, 0);
+        if (e != cudaSuccess) rs = cuda_fail(e, "capturing the step graph");
+    }
+    const int64_t per_replay = use_graph && graph.g ? graph_kernel_nodes(graph.g) : 0;
     while (rs == FRICP_OK) {
         if (use_graph) {
             e = cudaGraphLaunch(graph.exec, s);
