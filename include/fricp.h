@@ -306,7 +306,8 @@ typedef struct fricp_server fricp_server;
  * of the free device memory): a request's own buffers (28 B per source point,
  * 224 B per 256 points and one solver state of a few KB) and the index of its
  * target (16 B per point, 16 more with normals, 128 B per bucket of 16 for its
- * axis-aligned and oriented boxes, 8 B per point of FP16 storage), a target
+ * axis-aligned and oriented boxes, 8 B per point of FP16 storage; the oriented
+ * boxes of larger patches, 10 B per bucket, are not counted), a target
  * counted once however many requests in
  * flight share it. Requests are admitted in FIFO order while a slot is free
  * and the budget holds them. max_slots: requests in flight at most

@@ -379,7 +379,7 @@ __global__ void k_level_obb(const float4 *__restrict__ nodes, int L, int size, i
 // with normals, the median of the six distances to the point's tangent plane
 // (Sec. 5); the median of six is the mean of the 3rd and 4th smallest.
 //
-// One warp per query point, the traversal of warp_nn: the query's own bucket
+// One warp per query point (tiny targets and ties): the query's own bucket
 // is scanned first, then the siblings of its path to the root and what they
 // open, two tree levels per round; lanes test boxes and bucket points in
 // parallel. Pruning is in float: a box or candidate is skipped only when its
