@@ -307,7 +307,8 @@ typedef struct fricp_server fricp_server;
  * 224 B per 256 points and one solver state of a few KB) and the index of its
  * target (16 B per point, 16 more with normals, 128 B per bucket of 16 for its
  * axis-aligned and oriented boxes, 8 B per point of FP16 storage; the oriented
- * boxes of larger patches, 10 B per bucket, are not counted), a target
+ * boxes of larger patches, 10 B per bucket, and those of FP16 storage, 74 B
+ * per bucket, are not counted), a target
  * counted once however many requests in
  * flight share it. Requests are admitted in FIFO order while a slot is free
  * and the budget holds them. max_slots: requests in flight at most

@@ -33,7 +33,7 @@ using namespace fricp::host;
 thread_local std::string g_err;
 
 void free_target(TargetDev *t, cudaStream_t s) {
-    for (void *p : {(void *)t->pts, (void *)t->nrm, (void *)t->nodes, (void *)t->pts16})
+    for (void *p : {(void *)t->pts, (void *)t->nrm, (void *)t->nodes, (void *)t->pts16, (void *)t->obb16})
         if (p) cudaFreeAsync(p, s);
 }
 

@@ -1631,6 +1631,29 @@ cudaError_t morton_order(const float *x, int64_t n, const BoxPartial *box, cudaS
     return cudaGetLastError();
 }
 
+// Oriented boxes of all the levels of the walk, of points in the buckets of `nodes`.
+size_t oriented_boxes(int L) { return (size_t)((wide_leaf(L) + L + 7) / 8) * 8; }
+
+void launch_oriented(const float4 *pts, int64_t n, int L, const float4 *nodes, float4 *obb, cudaStream_t s) {
+    k_leaf_obb<<<(L + 127) / 128, 128, 0, s>>>(pts, n, L, obb);
+    counters().launches += 1;
+    const int first = wide_first(L);
+    for (int shift = 3; (L >> shift) >= first; shift += 3) {
+        const int size = L >> shift;
+        if (shift == 3)
+            k_patch_obb<32><<<(size + 7) / 8, 256, 0, s>>>(pts, n, L, shift, nodes, obb);
+        else if (shift <= 9)
+            k_patch_obb<256><<<size, 256, 0, s>>>(pts, n, L, shift, nodes, obb);
+        else
+            k_level_obb<<<(size + 127) / 128, 128, 0, s>>>(nodes, L, size, 0, obb);
+        counters().launches += 1;
+    }
+    if (first < 8) {
+        k_level_obb<<<1, 32, 0, s>>>(nodes, L, 0, 8 - first, obb);
+        counters().launches += 1;
+    }
+}
+
 }  // namespace
 
 cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cudaStream_t s, TargetDev *t,
@@ -1666,32 +1689,17 @@ cudaError_t build_target(const float *q_dev, const float *n_dev, int64_t n, cuda
     }
     e = pool_alloc(&t->pts, sizeof(float4) * n, s);
     if (e == cudaSuccess && n_dev) e = pool_alloc(&t->nrm, sizeof(float4) * n, s);
-    if (e == cudaSuccess) e = pool_alloc(&t->nodes, sizeof(float4) * 4 * ((size_t)L + ((wide_leaf(L) + L + 7) / 8) * 8), s);
+    if (e == cudaSuccess) e = pool_alloc(&t->nodes, sizeof(float4) * 4 * ((size_t)L + oriented_boxes(L)), s);
     if (e == cudaSuccess) {
         t->obb = t->nodes + 4 * (size_t)L;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q_dev, n_dev, order, n, t->pts, t->nrm);
         k_boxes<true><<<(L + 255) / 256, 256, 0, s>>>(t->pts, n, L, t->nodes);
-        k_leaf_obb<<<(L + 127) / 128, 128, 0, s>>>(t->pts, n, L, t->obb);
-        counters().launches += 3;
+        counters().launches += 2;
         for (int size = L / 256; size > 1; size /= 256) {
             k_boxes<false><<<(size + 255) / 256, 256, 0, s>>>(t->pts, n, size, t->nodes);
             counters().launches += 1;
         }
-        const int first = wide_first(L);
-        for (int shift = 3; (L >> shift) >= first; shift += 3) {
-            const int size = L >> shift;
-            if (shift == 3)
-                k_patch_obb<32><<<(size + 7) / 8, 256, 0, s>>>(t->pts, n, L, shift, t->nodes, t->obb);
-            else if (shift <= 9)
-                k_patch_obb<256><<<size, 256, 0, s>>>(t->pts, n, L, shift, t->nodes, t->obb);
-            else
-                k_level_obb<<<(size + 127) / 128, 128, 0, s>>>(t->nodes, L, size, 0, t->obb);
-            counters().launches += 1;
-        }
-        if (first < 8) {
-            k_level_obb<<<1, 32, 0, s>>>(t->nodes, L, 0, 8 - first, t->obb);
-            counters().launches += 1;
-        }
+        launch_oriented(t->pts, n, L, t->nodes, t->obb, s);
         e = cudaGetLastError();
     }
     cudaFreeAsync(order, s);
@@ -1718,19 +1726,37 @@ __global__ void k_encode16(const float4 *__restrict__ pts, const float4 *__restr
                           __half_as_ushort(__float2half_rn(uz)), 0);
 }
 
+// The points as the search decodes them.
+__global__ void k_decode16(Index ix, float4 *__restrict__ out) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < ix.n) out[j] = target_point<PREC_FP16>(ix, j);
+}
+
 cudaError_t build_fp16_storage(TargetDev *t, cudaStream_t s) {
     if (t->pts16) return cudaSuccess;
     ushort4 *p = nullptr;
+    float4 *obb = nullptr, *dec = nullptr;
     cudaError_t e = pool_alloc(&p, sizeof(ushort4) * (size_t)t->n, s);
-    if (e != cudaSuccess) return e;
-    k_encode16<<<(unsigned)((t->n + 255) / 256), 256, 0, s>>>(t->pts, t->nodes, (int)t->n, t->L, p);
-    counters().launches += 1;
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = pool_alloc(&obb, sizeof(float4) * 4 * oriented_boxes(t->L), s);
+    if (e == cudaSuccess) e = pool_alloc(&dec, sizeof(float4) * (size_t)t->n, s);
+    if (e == cudaSuccess) {
+        const unsigned nb = (unsigned)((t->n + 255) / 256);
+        k_encode16<<<nb, 256, 0, s>>>(t->pts, t->nodes, (int)t->n, t->L, p);
+        Index ix = make_index(*t);
+        ix.pts16 = p;
+        k_decode16<<<nb, 256, 0, s>>>(ix, dec);
+        counters().launches += 2;
+        launch_oriented(dec, t->n, t->L, t->nodes, obb, s);
+        e = cudaGetLastError();
+    }
+    if (dec) cudaFreeAsync(dec, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
-        cudaFreeAsync(p, s);
+        if (p) cudaFreeAsync(p, s);
+        if (obb) cudaFreeAsync(obb, s);
         return e;
     }
+    t->obb16 = obb;
     t->pts16 = p;
     return cudaSuccess;
 }
