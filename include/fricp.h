@@ -176,8 +176,8 @@ fricp_status fricp_target_create(const float *q_xyz, const float *q_normals, int
 fricp_status fricp_estimate_normals(const float *q_xyz, int64_t n, int32_t k, int32_t on_device,
                                     const double *viewpoint, float *normals_out, void *stream);
 
-/* Release a target (NULL is accepted). Waits for work queued on the target's
- * creation stream. */
+/* Release a target (NULL is accepted). Waits for all work queued on the device
+ * it was created on, whichever device is current. */
 fricp_status fricp_target_destroy(fricp_target *target);
 
 /* Number of points / whether normals are present. */

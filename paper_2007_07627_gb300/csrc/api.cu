@@ -16,6 +16,7 @@ using fricp::TargetDev;
 
 struct fricp_target {
     TargetDev d;
+    int device;   // the device that was current when it was built: its memory and everything that reads it are there
 };
 
 namespace fricp {
@@ -268,6 +269,8 @@ fricp_status fricp_target_create(const float *q_xyz, const float *q_normals, int
     fricp_target *t = new (std::nothrow) fricp_target;
     if (!t) return fail(FRICP_ENOMEM, "host allocation");
     std::memset(&t->d, 0, sizeof(t->d));
+    t->device = 0;
+    cudaGetDevice(&t->device);
     int bad = 0;
     cudaError_t e = fricp::build_target(q.ptr, q_normals ? nq.ptr : nullptr, n, ord.work, &t->d, &bad);
     if (e != cudaSuccess || bad) {
@@ -322,8 +325,17 @@ fricp_status fricp_estimate_normals(const float *q_xyz, int64_t n, int32_t k, in
 
 fricp_status fricp_target_destroy(fricp_target *t) {
     if (t == nullptr) return FRICP_OK;
+    // What is freed may be handed out again at once, so the target's own device is
+    // waited for, whichever is current, and the free is on a stream of that device:
+    // this thread's work stream, or the default one if that lives elsewhere.
+    cudaStream_t s = work_stream();
+    int cur = t->device, on = -1;
+    cudaGetDevice(&cur);
+    if (cur != t->device) cudaSetDevice(t->device);
     cudaDeviceSynchronize();
-    free_target(&t->d, work_stream());
+    if (cudaStreamGetDevice(s, &on) != cudaSuccess || on != t->device) s = nullptr;
+    free_target(&t->d, s);
+    if (cur != t->device) cudaSetDevice(cur);
     delete t;
     return FRICP_OK;
 }
