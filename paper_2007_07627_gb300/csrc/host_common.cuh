@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "fricp_internal.cuh"
+#include "launch_count.cuh"
 #include "linalg.cuh"
 #include "solver.cuh"
 
@@ -164,20 +165,6 @@ inline void to_caller(const double Tn[12], double s, const double c[3], double R
         const double Rc = Tn[3 * r] * c[0] + Tn[3 * r + 1] * c[1] + Tn[3 * r + 2] * c[2];
         t[r] = Tn[9 + r] / s + c[r] - Rc;
     }
-}
-
-// Kernel nodes of a captured graph (what one replay launches).
-inline int64_t graph_kernel_nodes(cudaGraph_t g) {
-    size_t n = 0;
-    if (cudaGraphGetNodes(g, nullptr, &n) != cudaSuccess || n == 0) return 0;
-    std::vector<cudaGraphNode_t> nodes(n);
-    if (cudaGraphGetNodes(g, nodes.data(), &n) != cudaSuccess) return 0;
-    int64_t k = 0;
-    for (size_t i = 0; i < n; ++i) {
-        cudaGraphNodeType ty;
-        if (cudaGraphNodeGetType(nodes[i], &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel) ++k;
-    }
-    return k;
 }
 
 struct Graph {

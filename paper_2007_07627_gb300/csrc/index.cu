@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "fricp_internal.cuh"
+#include "launch_count.cuh"
 
 namespace fricp {
 
@@ -1569,34 +1570,21 @@ cudaError_t wait_box(BoxPartial *res) {
     return e;
 }
 
-// Kernels one sort of n keys launches, for the launch counter: read off a capture
-// of the same call, which is not run, when n changes.
+// Kernels one sort of n keys launches, for the launch counter (0 if unknown: the
+// stream cannot be captured). A call whose size lies outside the ranges seen costs a
+// capture of the sort, 5 us (eval_pass on 2,000 and 1,999 points in turn: 144 us,
+// 139 us with one size).
 int64_t sort_launches(void *tmp, size_t tb, unsigned *code, unsigned *code2, int *idx, int *idx2, int n,
                       cudaStream_t s) {
-    thread_local int last_n = -1;
-    thread_local int64_t last = 0;
-    if (n == last_n) return last;
-    cudaGraph_t g = nullptr;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return 0;
-    const cudaError_t es = cub::DeviceRadixSort::SortPairs(tmp, tb, code, code2, idx, idx2, n, 0, 30, s);
-    if (cudaStreamEndCapture(s, &g) != cudaSuccess || es != cudaSuccess) {
-        cudaGetLastError();
-        if (g) cudaGraphDestroy(g);
-        return 0;
+    thread_local host::LaunchMemo memo;
+    int64_t k = memo.find(n);
+    if (k < 0) {
+        k = host::captured_kernels(s, [&] {
+            return cub::DeviceRadixSort::SortPairs(tmp, tb, code, code2, idx, idx2, n, 0, 30, s);
+        });
+        if (k >= 0) memo.add(n, k);
     }
-    size_t nn = 0;
-    cudaGraphGetNodes(g, nullptr, &nn);
-    std::vector<cudaGraphNode_t> nodes(nn);
-    if (nn) cudaGraphGetNodes(g, nodes.data(), &nn);
-    int64_t k = 0;
-    for (size_t i = 0; i < nn; ++i) {
-        cudaGraphNodeType ty;
-        if (cudaGraphNodeGetType(nodes[i], &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel) ++k;
-    }
-    cudaGraphDestroy(g);
-    last_n = n;
-    last = k;
-    return k;
+    return k > 0 ? k : 0;
 }
 
 // Morton order of n points: returns the permutation (device, caller frees).
