@@ -305,12 +305,11 @@ typedef struct fricp_server fricp_server;
 /* hbm_budget: bytes of device memory the requests in flight may hold (0 = half
  * of the free device memory): a request's own buffers (28 B per source point,
  * 224 B per 256 points and one solver state of a few KB) and the index of its
- * target (16 B per point, 16 more with normals, 128 B per bucket of 16 for its
- * axis-aligned and oriented boxes, 8 B per point of FP16 storage; the oriented
- * boxes of larger patches, 10 B per bucket, and those of FP16 storage, 74 B
- * per bucket, are not counted), a target
- * counted once however many requests in
- * flight share it. Requests are admitted in FIFO order while a slot is free
+ * target (16 B per point, 16 more with normals, 64 B per bucket of 16, their
+ * number rounded up to a power of two, for its axis-aligned boxes and about 73 B
+ * for the oriented ones; FP16 storage 8 B per point and about 73 B per bucket
+ * more), a target counted once however many requests in flight share it.
+ * Requests are admitted in FIFO order while a slot is free
  * and the budget holds them. max_slots: requests in flight at most
  * (1..4096). steps_per_sync: device steps per graph replay. max_queue:
  * requests waiting for admission at most. stream: submits of device sources

@@ -774,12 +774,14 @@ struct fricp_server {
 
 namespace {
 
-// Device bytes of a target's index: points, normals, box tree, oriented bucket boxes and (once built)
-// the FP16 storage.
-size_t target_bytes(const fricp_target *t) {
+// Device bytes of a target's index: points, normals, axis-aligned box tree, oriented
+// boxes of every level, and, once built or with `fp16` as if it were, the FP16
+// storage: offsets and oriented boxes of its own.
+size_t target_bytes(const fricp_target *t, bool fp16 = false) {
     const TargetDev &d = *fricp::target_dev(t);
-    size_t b = sizeof(float4) * (size_t)d.n * (d.has_normals ? 2 : 1) + sizeof(float4) * 8 * (size_t)d.L;
-    if (d.pts16) b += sizeof(ushort4) * (size_t)d.n;
+    const size_t boxes = sizeof(float4) * 4 * fricp::oriented_boxes(d.L);
+    size_t b = sizeof(float4) * (size_t)d.n * (d.has_normals ? 2 : 1) + sizeof(float4) * 4 * (size_t)d.L + boxes;
+    if (fp16 || d.pts16) b += sizeof(ushort4) * (size_t)d.n + boxes;
     return b;
 }
 
@@ -788,11 +790,8 @@ size_t target_bytes(const fricp_target *t) {
 // counted as if it will be built).
 size_t admission_bytes(const fricp_server *sv, const Request &rq) {
     size_t b = rq.bytes;
-    if (sv->targets.find(rq.target) == sv->targets.end()) {
-        b += target_bytes(rq.target);
-        if (rq.prm.precision == FRICP_PREC_FP16_STORAGE && fricp::target_dev(rq.target)->pts16 == nullptr)
-            b += sizeof(ushort4) * (size_t)fricp::target_dev(rq.target)->n;
-    }
+    if (sv->targets.find(rq.target) == sv->targets.end())
+        b += target_bytes(rq.target, rq.prm.precision == FRICP_PREC_FP16_STORAGE);
     return b;
 }
 

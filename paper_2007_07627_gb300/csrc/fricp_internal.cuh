@@ -423,6 +423,8 @@ FRICP_HD inline int wide_first(int L) {
 FRICP_HD inline int wide_pos(int first, int level_size) { return (level_size - first) / 7 + 8 - first; }
 FRICP_HD inline int wide_leaf(int L) { return wide_pos(wide_first(L), L); }
 FRICP_HD inline int wide_child(int first, int p) { return 8 * p + 8 * first - 56; }
+// Oriented boxes stored for L buckets: those of all levels, rounded up to eights.
+inline size_t oriented_boxes(int L) { return (size_t)((wide_leaf(L) + L + 7) / 8) * 8; }
 
 // Walk the tree for the point x = xh + xl of this group, offering every point of
 // every bucket within `bound` to `offer(j, p)`, which returns the smallest float

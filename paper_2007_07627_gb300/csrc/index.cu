@@ -1620,8 +1620,6 @@ cudaError_t morton_order(const float *x, int64_t n, const BoxPartial *box, cudaS
 }
 
 // Oriented boxes of all the levels of the walk, of points in the buckets of `nodes`.
-size_t oriented_boxes(int L) { return (size_t)((wide_leaf(L) + L + 7) / 8) * 8; }
-
 void launch_oriented(const float4 *pts, int64_t n, int L, const float4 *nodes, float4 *obb, cudaStream_t s) {
     k_leaf_obb<<<(L + 127) / 128, 128, 0, s>>>(pts, n, L, obb);
     counters().launches += 1;
