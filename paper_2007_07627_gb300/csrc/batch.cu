@@ -796,21 +796,21 @@ size_t admission_bytes(const fricp_server *sv, const Request &rq) {
 }
 
 // Admission of the queue's head requests that fit (FIFO, a free slot and room
-// in the budget): heavy work on s_admit, then the commit of each one on s_step
+// in the budget; with nothing in flight the head is admitted whatever it takes: it
+// was within the budget when it was submitted, its target may have gained FP16
+// storage since, and nothing else would ever make room): heavy work on s_admit, then the commit of each one on s_step
 // (after everything already queued there).
 fricp_status admit_queued(fricp_server *sv, int *admitted) {
     *admitted = 0;
     while (!sv->queue.empty()) {
         Request &rq = sv->queue.front();
         const size_t need = admission_bytes(sv, rq);
-        if (sv->used + need > sv->budget) break;
-        int slot = -1;
-        for (int p = 0; p < sv->max_slots; ++p)
-            if (!sv->slots[p]) {
-                slot = p;
-                break;
-            }
-        if (slot < 0) break;
+        int slot = -1, flying = 0;
+        for (int p = sv->max_slots - 1; p >= 0; --p) {
+            if (sv->slots[p]) ++flying;
+            else slot = p;
+        }
+        if (slot < 0 || (flying > 0 && sv->used + need > sv->budget)) break;
         auto run = std::make_unique<Running>();
         run->req = std::move(rq);
         sv->queue.pop_front();
@@ -950,7 +950,7 @@ extern "C" fricp_status fricp_server_submit(fricp_server *sv, const fricp_target
     r.has_T0 = T0 != nullptr;
     if (T0) std::memcpy(r.T0, T0, sizeof(r.T0));
     r.bytes = PairBuffers::need(m, 0);
-    if (r.bytes + target_bytes(target) > sv->budget)
+    if (r.bytes + target_bytes(target, r.prm.precision == FRICP_PREC_FP16_STORAGE) > sv->budget)
         return fail(FRICP_EINVAL, "request and its target need more device memory than the server budget");
     if (on_device) {
         cudaError_t e = cudaEventRecord(sv->ev_user, sv->user);

@@ -79,3 +79,33 @@ def test_oriented_boxes_of_every_level_and_storage_count(fr, pair, precision):
     assert r is not None and r["status"] == "OK"
     srv.destroy()
     t.destroy()
+
+
+def test_fp16_request_over_the_budget_is_refused_at_submit(fr, pair):
+    """Accepted without its storage counted, it would wait at the head of the queue for ever."""
+    Q, P = pair
+    t = fr.target_create(Q)
+    srv = fr.Server(hbm_budget=REQUEST + INDEX + FP16 // 2, max_slots=2)
+    with pytest.raises(fr.FricpError) as ei:
+        srv.submit(t, P, _prm(fr, "fp16"))
+    assert "budget" in str(ei.value)
+    (r,), _ = _serve(srv, [srv.submit(t, P, _prm(fr))])
+    assert r is not None and r["status"] == "OK"
+    srv.destroy()
+    t.destroy()
+
+
+def test_accepted_request_is_served_although_its_target_has_grown(fr, pair):
+    """FP16 storage built between submit and admission takes the target over the budget."""
+    Q, P = pair
+    t = fr.target_create(Q)
+    srv = fr.Server(hbm_budget=REQUEST + INDEX + STATE, max_slots=2)
+    tickets = [srv.submit(t, P, _prm(fr)), srv.submit(t, P, _prm(fr))]
+    fr.register(t, P, params=_prm(fr, "fp16"))
+    res, most = _serve(srv, tickets)
+    assert most == 1
+    alone = fr.register(t, P, params=_prm(fr))
+    for r in res:
+        assert r is not None and r["status"] == "OK" and np.array_equal(r["R"], alone["R"])
+    srv.destroy()
+    t.destroy()
