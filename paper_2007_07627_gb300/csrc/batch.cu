@@ -785,14 +785,14 @@ size_t target_bytes(const fricp_target *t, bool fp16 = false) {
     return b;
 }
 
-// Bytes a request adds to the budget in use: its own buffers, and its target's
-// index unless a request in flight already holds that target (FP16 storage is
-// counted as if it will be built).
+// Bytes a request adds to the budget in use: its own buffers, and of its target's
+// index (FP16 storage counted if built or if this request will have it built) what
+// the requests in flight on that target have not been charged for.
 size_t admission_bytes(const fricp_server *sv, const Request &rq) {
-    size_t b = rq.bytes;
-    if (sv->targets.find(rq.target) == sv->targets.end())
-        b += target_bytes(rq.target, rq.prm.precision == FRICP_PREC_FP16_STORAGE);
-    return b;
+    const size_t index = target_bytes(rq.target, rq.prm.precision == FRICP_PREC_FP16_STORAGE);
+    const auto it = sv->targets.find(rq.target);
+    const size_t charged = it == sv->targets.end() ? 0 : it->second.second;
+    return rq.bytes + (index > charged ? index - charged : 0);
 }
 
 // Admission of the queue's head requests that fit (FIFO, a free slot and room
@@ -843,7 +843,8 @@ fricp_status admit_queued(fricp_server *sv, int *admitted) {
         r.host_pts.clear();
         r.host_pts.shrink_to_fit();
         auto &tr = sv->targets[r.target];
-        if (tr.first++ == 0) tr.second = need - r.bytes;
+        ++tr.first;
+        tr.second += need - r.bytes;
         sv->used += need;
         sv->slots[slot] = std::move(run);
         ++*admitted;

@@ -41,11 +41,11 @@ def _prm(fr, precision="fp64"):
     return fr.params_default("p2p", precision=precision, max_iters=5)
 
 
-def _serve(srv, tickets, steps=400):
+def _serve(srv, tickets, nsteps=8, steps=400):
     """Results of the tickets; None for those that have not finished after `steps` server steps."""
     res, most = {}, 0
     for _ in range(steps):
-        flying, _ = srv.step(8)
+        flying, _ = srv.step(nsteps)
         most = max(most, flying)
         for t in tickets:
             r = srv.poll(t) if t not in res else None
@@ -107,5 +107,18 @@ def test_accepted_request_is_served_although_its_target_has_grown(fr, pair):
     alone = fr.register(t, P, params=_prm(fr))
     for r in res:
         assert r is not None and r["status"] == "OK" and np.array_equal(r["R"], alone["R"])
+    srv.destroy()
+    t.destroy()
+
+
+@pytest.mark.parametrize("room,together", [(FP16 - REQUEST // 2, 1), (FP16, 2)])
+def test_storage_built_for_a_target_in_flight_is_charged(fr, pair, room, together):
+    """An FP16 request joins an FP64 one on the same target only when the storage fits too."""
+    Q, P = pair
+    t = fr.target_create(Q)
+    srv = fr.Server(hbm_budget=2 * (REQUEST + STATE) + INDEX + room, max_slots=2, steps_per_sync=1)
+    prms = [fr.params_default("p2p", precision=p, max_iters=100, eps=1e-14) for p in ("fp64", "fp16")]
+    res, most = _serve(srv, [srv.submit(t, P, prm) for prm in prms], nsteps=1)
+    assert most == together and all(r is not None and r["status"] == "OK" for r in res)
     srv.destroy()
     t.destroy()
