@@ -303,7 +303,8 @@ void fricp_batch_last_shape(int32_t *chunk, int32_t *search_blocks_per_sm,
 typedef struct fricp_server fricp_server;
 
 /* hbm_budget: bytes of device memory the requests in flight may hold (0 = half
- * of the free device memory): a request's own buffers (28 B per source point,
+ * of the free device memory, what the library's pool keeps unused included; no
+ * more than all of it): a request's own buffers (28 B per source point,
  * 224 B per 256 points and one solver state of a few KB) and the index of its
  * target (16 B per point, 16 more with normals, 64 B per bucket of 16, their
  * number rounded up to a power of two, for its axis-aligned boxes and about 73 B

@@ -211,6 +211,17 @@ cudaError_t pool_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     return e;
 }
 
+size_t pool_idle_bytes() {
+    const cudaMemPool_t pool = device_pool();
+    uint64_t reserved = 0, used = 0;
+    if (pool == nullptr || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return reserved > used ? (size_t)(reserved - used) : 0;
+}
+
 const TargetDev *target_dev(const fricp_target *t) { return t ? &t->d : nullptr; }
 void set_last_error(const char *msg) { g_err = msg; }
 }  // namespace fricp

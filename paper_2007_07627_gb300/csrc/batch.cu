@@ -908,6 +908,7 @@ extern "C" fricp_status fricp_server_create(size_t hbm_budget, int32_t max_slots
     size_t free_b = 0, total_b = 0;
     cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
     if (e != cudaSuccess) return cuda_fail(e, "querying device memory");
+    free_b += fricp::pool_idle_bytes();   // the requests' buffers come from the pool
     if (hbm_budget == 0) hbm_budget = free_b / 2;
     if (hbm_budget > free_b) return fail(FRICP_EINVAL, "hbm_budget exceeds free device memory");
     auto sv = std::make_unique<fricp_server>();

@@ -122,3 +122,16 @@ def test_storage_built_for_a_target_in_flight_is_charged(fr, pair, room, togethe
     assert most == together and all(r is not None and r["status"] == "OK" for r in res)
     srv.destroy()
     t.destroy()
+
+
+def test_memory_the_pool_keeps_is_free_to_a_server(fr):
+    """What a destroyed target held and the pool kept is the server's to use."""
+    import torch
+    g = np.random.default_rng(4)
+    fr.target_create(g.random((2_000_000, 3)).astype(np.float32)).destroy()   # index and sort: over 100 MB
+    free, total = torch.cuda.mem_get_info()
+    srv = fr.Server(hbm_budget=free + (32 << 20), max_slots=2)
+    srv.destroy()
+    with pytest.raises(fr.FricpError) as ei:
+        fr.Server(hbm_budget=total + (1 << 30), max_slots=2)
+    assert "free device memory" in str(ei.value)
