@@ -247,9 +247,7 @@ __global__ void k_leaf_obb(const float4 *__restrict__ pts, int64_t n, int L, flo
 }
 
 // Oriented boxes of the patches three, six and nine levels above the buckets (128,
-// 1,024 and 8,192 points), one per NT threads: axes of the points' scatter about the
-// axis-aligned box's middle, extents about a float centre, widened as obb_fit's.
-// `shift` = 3, 6 or 9.
+// 1,024 and 8,192 points), one per NT threads (obb_fit_patch). `shift` = 3, 6 or 9.
 template <int NT>
 __global__ void __launch_bounds__(256) k_patch_obb(const float4 *__restrict__ pts, int64_t n, int L, int shift,
                                                    const float4 *__restrict__ nodes, float4 *__restrict__ obb) {
@@ -289,59 +287,14 @@ __global__ void __launch_bounds__(256) k_patch_obb(const float4 *__restrict__ pt
         c[1] = 0.5f * lo.y + 0.5f * hi.y;
         c[2] = 0.5f * lo.z + 0.5f * hi.z;
     }
-    float v[9] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    for (int k = tid; k < cnt; k += NT) {
-        const float4 p = pts[beg + k];
-        const float d[3] = {p.x - c[0], p.y - c[1], p.z - c[2]};
-        v[0] += d[0];
-        v[1] += d[1];
-        v[2] += d[2];
-        v[3] = fmaf(d[0], d[0], v[3]);
-        v[4] = fmaf(d[0], d[1], v[4]);
-        v[5] = fmaf(d[0], d[2], v[5]);
-        v[6] = fmaf(d[1], d[1], v[6]);
-        v[7] = fmaf(d[1], d[2], v[7]);
-        v[8] = fmaf(d[2], d[2], v[8]);
-    }
-    fold(v, 9, false);
-    const float ic = 1.0f / fmaxf((float)cnt, 1.0f);
-    const float xy = v[4] - v[0] * v[1] * ic, xz = v[5] - v[0] * v[2] * ic, yz = v[7] - v[1] * v[2] * ic;
-    float A[3][3] = {{v[3] - v[0] * v[0] * ic, xy, xz}, {xy, v[6] - v[1] * v[1] * ic, yz},
-                     {xz, yz, v[8] - v[2] * v[2] * ic}};
-    float a[3][3];
-    obb_axes(A, a);
-    float e[6] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max u, max -u
-    for (int k = tid; k < cnt; k += NT) {
-        const float4 p = pts[beg + k];
-        const float d[3] = {p.x - c[0], p.y - c[1], p.z - c[2]};
-        for (int r = 0; r < 3; ++r) {
-            const float u = fmaf(a[r][2], d[2], fmaf(a[r][1], d[1], a[r][0] * d[0]));
-            e[r] = fmaxf(e[r], u);
-            e[3 + r] = fmaxf(e[3 + r], -u);
-        }
-    }
-    fold(e, 6, true);
-    if (cnt > 0) {   // the middle of the extents
-        const float m[3] = {0.5f * (e[0] - e[3]), 0.5f * (e[1] - e[4]), 0.5f * (e[2] - e[5])};
-        for (int r = 0; r < 3; ++r) c[r] += fmaf(m[2], a[2][r], fmaf(m[1], a[1][r], m[0] * a[0][r]));
-    }
-    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // half-extents and radius^2 about the float centre
-    for (int k = tid; k < cnt; k += NT) {
-        const float4 p = pts[beg + k];
-        const float d[3] = {p.x - c[0], p.y - c[1], p.z - c[2]};
-        for (int r = 0; r < 3; ++r) h[r] = fmaxf(h[r], fabsf(fmaf(a[r][2], d[2], fmaf(a[r][1], d[1], a[r][0] * d[0]))));
-        h[3] = fmaxf(h[3], fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0])));
-    }
-    fold(h, 4, true);
+    float4 box[4];
+    obb_fit_patch(pts + beg, cnt, c, tid, NT, fold, box);
     if (!in || tid != 0) return;
     if (cnt == 0) {
         empty_obb(o);
         return;
     }
-    const float r = sqrtf(h[3]) * (1.0f + 1e-6f);
-    for (int k = 0; k < 3; ++k) h[k] = obb_widen(h[k], r);
-    o[0] = make_float4(c[0], c[1], c[2], h[0]);
-    for (int k = 0; k < 3; ++k) o[8 + 8 * k] = make_float4(a[k][0], a[k][1], a[k][2], k == 0 ? h[1] : (k == 1 ? h[2] : r));
+    for (int k = 0; k < 4; ++k) o[8 * k] = box[k];
 }
 
 // The levels above (few, large nodes): the axis-aligned box in the same form.

@@ -156,6 +156,65 @@ FRICP_HD inline void obb_fit(const float4 *p, int cnt, float4 out[4]) {
     out[3] = make_float4(ax[2][0], ax[2][1], ax[2][2], r);
 }
 
+// Oriented box of a patch of cnt >= 0 points, in the same form, by a team of nt
+// threads: thread t takes points t, t + nt, ... and fold(v, k, max) leaves the sum
+// (or maximum) of v[0 .. k) over the team in all of them. Axes of the points'
+// scatter about c0 (the middle of their axis-aligned box), extents and radius about
+// the middle of the extents, widened as obb_fit's. Nothing of a patch without points
+// is used.
+template <class Fold>
+FRICP_HD inline void obb_fit_patch(const float4 *p, int cnt, const float c0[3], int t, int nt, Fold fold,
+                                   float4 out[4]) {
+    float c[3] = {c0[0], c0[1], c0[2]};
+    float v[9] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    for (int k = t; k < cnt; k += nt) {
+        const float d[3] = {p[k].x - c[0], p[k].y - c[1], p[k].z - c[2]};
+        v[0] += d[0];
+        v[1] += d[1];
+        v[2] += d[2];
+        v[3] = fmaf(d[0], d[0], v[3]);
+        v[4] = fmaf(d[0], d[1], v[4]);
+        v[5] = fmaf(d[0], d[2], v[5]);
+        v[6] = fmaf(d[1], d[1], v[6]);
+        v[7] = fmaf(d[1], d[2], v[7]);
+        v[8] = fmaf(d[2], d[2], v[8]);
+    }
+    fold(v, 9, false);
+    const float ic = 1.0f / fmaxf((float)cnt, 1.0f);
+    const float xy = v[4] - v[0] * v[1] * ic, xz = v[5] - v[0] * v[2] * ic, yz = v[7] - v[1] * v[2] * ic;
+    float A[3][3] = {{v[3] - v[0] * v[0] * ic, xy, xz}, {xy, v[6] - v[1] * v[1] * ic, yz},
+                     {xz, yz, v[8] - v[2] * v[2] * ic}};
+    float a[3][3];
+    obb_axes(A, a);
+    float e[6] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max u, max -u
+    for (int k = t; k < cnt; k += nt) {
+        const float d[3] = {p[k].x - c[0], p[k].y - c[1], p[k].z - c[2]};
+        for (int r = 0; r < 3; ++r) {
+            const float u = fmaf(a[r][2], d[2], fmaf(a[r][1], d[1], a[r][0] * d[0]));
+            e[r] = fmaxf(e[r], u);
+            e[3 + r] = fmaxf(e[3 + r], -u);
+        }
+    }
+    fold(e, 6, true);
+    if (cnt > 0) {   // the middle of the extents
+        const float m[3] = {0.5f * (e[0] - e[3]), 0.5f * (e[1] - e[4]), 0.5f * (e[2] - e[5])};
+        for (int r = 0; r < 3; ++r) c[r] += fmaf(m[2], a[2][r], fmaf(m[1], a[1][r], m[0] * a[0][r]));
+    }
+    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // half-extents and radius^2 about the float centre
+    for (int k = t; k < cnt; k += nt) {
+        const float d[3] = {p[k].x - c[0], p[k].y - c[1], p[k].z - c[2]};
+        for (int r = 0; r < 3; ++r) h[r] = fmaxf(h[r], fabsf(fmaf(a[r][2], d[2], fmaf(a[r][1], d[1], a[r][0] * d[0]))));
+        h[3] = fmaxf(h[3], fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0])));
+    }
+    fold(h, 4, true);
+    const float r = sqrtf(h[3]) * (1.0f + 1e-6f);
+    for (int k = 0; k < 3; ++k) h[k] = obb_widen(h[k], r);
+    out[0] = make_float4(c[0], c[1], c[2], h[0]);
+    out[1] = make_float4(a[0][0], a[0][1], a[0][2], h[1]);
+    out[2] = make_float4(a[1][0], a[1][1], a[1][2], h[2]);
+    out[3] = make_float4(a[2][0], a[2][1], a[2][2], r);
+}
+
 // Squared distance from x = xh + xl to the box (c, h0) (a0, h1) (a1, h2) (a2, .),
 // in float. Against the widening of obb_fit, the float rounding of
 // u = A ((xh - c) + xl) (at most ~5.2e-7 of |x - c| per axis) leaves the result
