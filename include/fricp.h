@@ -29,6 +29,9 @@
  *   - `stream` is a cudaStream_t (NULL = legacy default stream). All device work
  *     of a call is issued on it; calls that return results to the host wait for
  *     that stream only.
+ *   - Device memory comes from a pool of the library's own, one per device, which
+ *     keeps up to 256 MB of what is freed for its next calls (and gives it back
+ *     when an allocation of its own does not fit).
  *   - No call aborts, traps or exits. Every call returns a fricp_status; on any
  *     status other than FRICP_OK, fricp_last_error() returns a message
  *     (thread-local, valid until the next call on the same thread).
@@ -92,10 +95,9 @@ typedef enum {
     FRICP_PREC_FP16_STORAGE = 2
 } fricp_precision;
 
-/* Layout of the exact closest-point search (Eq. 3) of fricp_register. Both
- * values run the same search (eight lanes per query over the box tree, four
- * Morton-adjacent queries per warp), which is faster than either of the two
- * layouts they once chose between; the result is the exact argmin. */
+/* Accepted and ignored: both values run the one exact closest-point search
+ * (Eq. 3), which is faster than either of the two layouts they once chose
+ * between. */
 typedef enum {
     FRICP_SEARCH_TILE = 0,
     FRICP_SEARCH_QUERY = 1
@@ -104,7 +106,7 @@ typedef enum {
 /* Solver parameters. fricp_params_default fills the paper's defaults. */
 typedef struct {
     int32_t variant;            /* fricp_variant */
-    int32_t anderson_m;         /* m, previous iterates used by AA: 5 (Sec. 4.2). 0..8; 0 = plain MM */
+    int32_t anderson_m;         /* m, previous iterates used by AA: 5 (Sec. 4.2). 0..5; 0 = plain MM */
     int32_t max_iters;          /* I_nu for point-to-point: 1000 (Sec. 4.3). >= 1 */
     int32_t p2pl_iters_first;   /* I_nu at nu_max for point-to-plane: 6 (Sec. 5) */
     int32_t p2pl_iters_cap;     /* +1 per nu stage, at most 10 (Sec. 5) */
@@ -119,14 +121,15 @@ typedef struct {
     int32_t max_steps;          /* hard cap on device steps (correspondence passes): 100000 */
     double  timeout_s;          /* host wait limit for one registration: 600 */
     int32_t precision;          /* fricp_precision: FRICP_PREC_FP64 */
-    int32_t search;             /* fricp_search: FRICP_SEARCH_QUERY */
+    int32_t search;             /* fricp_search, ignored: FRICP_SEARCH_QUERY */
 } fricp_params;
 
 /* Result of one registration. All transforms in the caller's coordinates. */
 typedef struct {
     double  R[9];               /* row-major rotation */
     double  t[3];               /* translation */
-    int32_t status;             /* FRICP_OK, FRICP_EDEGENERATE or FRICP_EOVERFLOW */
+    int32_t status;             /* FRICP_OK or FRICP_EDEGENERATE; of a served request whose admission
+                                   failed, the status it failed with */
     int32_t iterations;         /* inner-loop bodies run over all nu stages (Alg. 1 / Alg. 2) */
     int32_t corr_passes;        /* correspondence computations the algorithm needed */
     int32_t aa_accepted;        /* Anderson iterates that passed the energy check */
@@ -278,7 +281,7 @@ fricp_status fricp_batch_register(int32_t npairs, const fricp_target *const *tar
  * search blocks per SM (clamped to the kernel's occupancy) and the ticket
  * order: 0 = from an atomic counter; 1 = dealt in a fixed stride; 2 = from the
  * counter with chunk = 8. A warp searches four queries of its ticket at a
- * time. chunk = 0 returns to autotuning. The results do not depend on the shape,
+ * time, so a chunk of 1 or 2 leaves lanes idle. chunk = 0 returns to autotuning. The results do not depend on the shape,
  * only the time. Errors: EINVAL. */
 fricp_status fricp_batch_set_shape(int32_t chunk, int32_t search_blocks_per_sm, int32_t static_order);
 

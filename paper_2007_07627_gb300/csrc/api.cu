@@ -98,6 +98,7 @@ fricp_status run_steps(const fricp::StepArgs &a, int variant, int ntiles, const 
     }
     // The GPU runs the first steps while the host captures the graph of the others
     // (a step past the end does nothing; small step budgets are kept to the step).
+    // Torus, 2,000 points: 1,874 -> 1,822 us, quartiles within 10 us, 4 x 40 runs a side.
     if (rs == FRICP_OK && use_graph && init_m == 0 && prm.max_steps >= 4096) {
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = fricp::launch_step(a, variant, prec, ntiles, s);
         if (e != cudaSuccess) rs = cuda_fail(e, "launching step");

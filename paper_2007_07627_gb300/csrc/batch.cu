@@ -444,10 +444,12 @@ class BatchEngine {
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         // (chunk, order): tickets of one or two rounds of kGroupQ queries from
-        // the counter, one round in a fixed stride (tickets of 16 and half the
-        // blocks were never the fastest: 16 mixed pairs, M 2k-200k, 169 ms per
-        // batch with tickets of 4, 176 with 8, 194 with 16, 173 in a stride, 197
-        // with half the blocks)
+        // the counter, one round in a fixed stride. ms per batch with tickets of
+        // 4, 8 and 16, of 4 in a stride, and of 4 on half the blocks: 16 mixed
+        // pairs, M 2k-200k, FP64 164, 173, 193, 166, 195; the same in FP32 122,
+        // 128, 148, 120, 141, in FP16 147, 152, 178, 148, 171; 6 pairs, M 1k-4k,
+        // 50.0, 53.8, 61.0, 48.5, 49.2. The order that wins hardly depends on the
+        // precision (1% at most), so one shape serves a size class in all of them.
         const int cands[][2] = {{kGroupQ, kOrderCounter}, {2 * kGroupQ, kOrderCounter}, {kGroupQ, kOrderStride}};
         BatchShape best{1, nn_max, acc_max, 0};
         float best_ms = 1e30f;

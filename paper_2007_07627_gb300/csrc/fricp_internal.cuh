@@ -391,14 +391,15 @@ constexpr int kWarpStack = 1024;  // walk stack of a warp in the neighbour kerne
 // points (ellipsoids, M = 200,000: 204 us a pass; on the axis-aligned boxes, which
 // hold both, about 600).
 //
-// What bounds it: issue slots (63% busy) and the L1 latency of each round's
-// loads; about 95 instructions a round and 60 a bucket, 16 rounds and 8 buckets
-// for four warm-started queries that stay together. Measured (ellipsoids,
+// What bounds it: issue slots (74% busy; about 95 instructions a round and 60 a
+// bucket, 16 rounds and 8 buckets for four warm-started queries that stay
+// together), then the L1 latency of each round's loads. Measured (ellipsoids,
 // N = 500,000, M = 200,000, FP64, mean over a registration's passes): two
-// queries per warp over the axis-aligned boxes 357 us, this 196 us; with four
-// lanes per query (two children each) 206 us, with two 364 us before the boxes
-// were stored in eights (the L1 then serves whole lines: 377 -> 335 us); the
-// oriented boxes above the buckets take the rounds per query from 20.5 to 14.8.
+// queries per warp over the axis-aligned boxes 357 us, this 157 us (196 us
+// before k_nn took the hard tickets first); with four lanes per query (two
+// children each) 172 us. On the way: storing the boxes in eights, so that the L1
+// serves whole lines, 377 -> 335 us; the oriented boxes above the buckets take
+// the rounds per query from 20.5 to 14.8.
 // ---------------------------------------------------------------------------
 constexpr int kGroup = 8;                         // lanes per query
 constexpr int kGroupQ = 32 / kGroup;              // queries per warp

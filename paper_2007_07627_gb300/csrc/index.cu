@@ -4,7 +4,8 @@
 // tree of axis-aligned boxes whose leaves are buckets of kLeaf consecutive
 // target points in Morton order. The tree is implicit (node i has children 2i
 // and 2i+1), so building it is: bounding box -> 30-bit Morton keys -> radix sort
-// -> gather into float4 -> leaf boxes -> one pass per tree level.
+// -> gather into float4 -> leaf boxes -> one launch per eight tree levels, and the
+// oriented boxes that the search walks (obb.cuh) for every third level.
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
@@ -565,8 +566,9 @@ __global__ void __launch_bounds__(kKnnBlock) k_knn6_stats(Index ix, double *__re
 // to k_knn6_rest, which gives each of its points a warp.
 // With every distance and comparison in FP64, and the left-over tiles searched
 // point by point by their own warp, the FP64 pipe and a few such warps were the
-// bound (ellipsoids, 500,000 points: 2.48 ms); now 0.36 ms, issue-bound, and 0.11
-// ms for the rest.
+// bound (ellipsoids, 500,000 points: 2.48 ms); now 0.34 ms, and 0.11 ms for the
+// rest. What bounds it: issue slots (55% busy, 17 of 32 lanes at work) and the
+// candidates' loads, with the busiest SM 30% above the average.
 constexpr int kKnnCand = 192;   // candidate buckets per tile
 
 __device__ __forceinline__ float box_box_d2(float4 alo, float4 ahi, float4 blo, float4 bhi) {
@@ -1056,7 +1058,8 @@ __global__ void __launch_bounds__(kKnnBlock) k_knn6_rest(Index ix, double *__res
 // GB300 issues an FP64 warp instruction once in 64 cycles however many lanes it
 // has, so FP64 work spread over a warp per point (distances, list comparisons,
 // covariance sums, 3.0 ms of k_knn_cov for 100,000 points) was the bound; with a
-// point per lane it is 1/32 of that, and the search is bound by issue slots.
+// point per lane it is 1/32 of that. The kernel now keeps 57% of the issue slots
+// and 33% of the FP64 pipe busy: the search's issue and latency are the bound.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double exact_d2(float4 q, const float xq[3]) {
     const double a0 = (double)q.x - (double)xq[0], a1 = (double)q.y - (double)xq[1], a2 = (double)q.z - (double)xq[2];
@@ -1525,8 +1528,9 @@ cudaError_t wait_box(BoxPartial *res) {
 
 // Kernels one sort of n keys launches, for the launch counter (0 if unknown: the
 // stream cannot be captured). A call whose size lies outside the ranges seen costs a
-// capture of the sort, 5 us (eval_pass on 2,000 and 1,999 points in turn: 144 us,
-// 139 us with one size).
+// capture of the sort (eval_pass on 20,000 and 19,999 points in turn, captured in
+// every call 205 us, in none 194 us; on 2,000 and 1,999, whose sort is two kernels,
+// 137 and 137 us).
 int64_t sort_launches(void *tmp, size_t tb, unsigned *code, unsigned *code2, int *idx, int *idx2, int n,
                       cudaStream_t s) {
     thread_local host::LaunchMemo memo;
