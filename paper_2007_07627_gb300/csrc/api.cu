@@ -223,6 +223,13 @@ size_t pool_idle_bytes() {
     return reserved > used ? (size_t)(reserved - used) : 0;
 }
 
+void pool_trim(cudaStream_t s) {
+    const cudaMemPool_t pool = device_pool();
+    if (pool == nullptr) return;
+    cudaStreamSynchronize(s);
+    cudaMemPoolTrimTo(pool, kPoolKeep);
+}
+
 const TargetDev *target_dev(const fricp_target *t) { return t ? &t->d : nullptr; }
 void set_last_error(const char *msg) { g_err = msg; }
 }  // namespace fricp
@@ -347,6 +354,7 @@ fricp_status fricp_target_destroy(fricp_target *t) {
     cudaDeviceSynchronize();
     if (cudaStreamGetDevice(s, &on) != cudaSuccess || on != t->device) s = nullptr;
     free_target(&t->d, s);
+    fricp::pool_trim(s);   // freed memory stays with the pool until something waits for its stream
     if (cur != t->device) cudaSetDevice(cur);
     delete t;
     return FRICP_OK;

@@ -1053,8 +1053,8 @@ extern "C" fricp_status fricp_server_destroy(fricp_server *sv) {
         if (r) r->buf.free(sv->s_step);
     for (auto &r : sv->queue)
         if (r.dev_pts) cudaFreeAsync(r.dev_pts, sv->s_step);
-    if (sv->s_step) cudaStreamSynchronize(sv->s_step);
     sv->eng.release();
+    if (sv->s_step) cudaStreamSynchronize(sv->s_step);   // the pool gives back what it need not keep
     if (sv->ev_admit) cudaEventDestroy(sv->ev_admit);
     if (sv->ev_user) cudaEventDestroy(sv->ev_user);
     if (sv->poll) cudaEventDestroy(sv->poll);
