@@ -223,9 +223,13 @@ size_t pool_idle_bytes() {
     return reserved > used ? (size_t)(reserved - used) : 0;
 }
 
-void pool_trim(cudaStream_t s) {
+// Once s has run, gives back what the current device's pool holds unused above kPoolKeep.
+static void pool_trim(cudaStream_t s) {
     const cudaMemPool_t pool = device_pool();
-    if (pool == nullptr) return;
+    uint64_t reserved = 0;
+    if (pool == nullptr || (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+                            reserved <= kPoolKeep))
+        return;
     cudaStreamSynchronize(s);
     cudaMemPoolTrimTo(pool, kPoolKeep);
 }

@@ -624,7 +624,6 @@ void set_last_error(const char *msg);
 // cudaFreeAsync; the pool keeps up to kPoolKeep bytes across synchronisations.
 constexpr size_t kPoolKeep = (size_t)256 << 20;
 cudaError_t pool_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
-void pool_trim(cudaStream_t s);   // waits for s, then gives back what the current device's pool holds above kPoolKeep
 size_t pool_idle_bytes();   // held by the current device's pool and in no use: not free to the driver, free to the library
 template <class T>
 inline cudaError_t pool_alloc(T **p, size_t bytes, cudaStream_t s) {
