@@ -789,6 +789,10 @@ __device__ __forceinline__ void near_scan(const Index &ix, const float xq[3], in
 // The point's bucket and its sibling are scanned first; then the walk of group_nn
 // over the oriented boxes, by the whole warp: up to four nodes a round, eight
 // children each, and the buckets within the bound two at a time, nearest first.
+// Squares below it lose bits to underflow, and the float distances their relative
+// error of 4e-7: such a list is left to FP64 (points about 1e-18 apart; also seven
+// copies of a point).
+constexpr float kNearMin = 1e-36f;
 constexpr int kNearStack = kWarpStack;   // a round replaces up to 4 nodes by at most 32: below 9 levels x 32 + 8
 
 __device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3], int skip, int K, float bound,
@@ -842,7 +846,7 @@ __device__ __forceinline__ int near_knn(const Index &ix, int i, const float xq[3
     const float kth = __shfl_sync(FULL, t.d, K - 1);
     const float next = K < 32 ? __shfl_sync(FULL, t.d, K & 31) : t.spill;
     t.bound = kth;
-    return !(kth < INF) || (next <= kth * kTieWindow && next < INF) ? 1 : 0;
+    return !(kth >= kNearMin && kth < INF) || (next <= kth * kTieWindow && next < INF) ? 1 : 0;
 }
 
 // The same selection by float distance: each lane keeps its seven nearest, sorted.
@@ -907,7 +911,7 @@ __device__ __forceinline__ int tile_near7(const Index &ix, int g, int i, bool li
         if (need)
             for (int j = beg; j < end; ++j) near7_offer(b, __ldg(ix.pts + j), xq, j);
     }
-    return __any_sync(FULL, live && !(b.d[6] > b.d[5] * kTieWindow && b.d[5] < INFINITY)) ? 1 : 0;
+    return __any_sync(FULL, live && !(b.d[6] > b.d[5] * kTieWindow && b.d[5] < INFINITY && b.d[5] >= kNearMin)) ? 1 : 0;
 }
 
 // Sort of six non-negative doubles by their bits (they order alike).
